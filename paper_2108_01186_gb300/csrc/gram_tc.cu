@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(288, 1) k_gram_async(const BlkDesc* __restrict
     const long long g_begin = (long long)blockIdx.x * kGChunk;
     if (g_begin >= B.G) return;
     const int nst = kSub / kGK;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = (int)tc_uniform((uint32_t)tid >> 5), lane = tid & 31;
     unsigned char* base =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(g_smem_raw) + 1023) & ~(uintptr_t)1023);
     unsigned char* tiles = base;                                  // kGStages x 3 bf16 tiles
@@ -298,33 +298,38 @@ __global__ void __launch_bounds__(288, 1) k_gram_async(const BlkDesc* __restrict
     const uint32_t dcross = tmem + (uint32_t)(2 * MN);
     bool ok = true;
     if (warp == 8) {
-        // ---- MMA issue (lane 0): per stage, six split products per 16-point K step
-        if (lane == 0) {
-            const uint32_t idesc = umma_idesc_bf16(kGRows, MN);
-            for (int st = 0; st < nst && ok; ++st) {
-                const int b = st & 1;
-                ok = tc_mbar_sleep_or_abort(&conv_full[b], (uint32_t)((st >> 1) & 1), &s_abort);
-                // per-stage accumulator b was read back (stage st - 2)
-                if (ok && st >= 2) ok = tc_mbar_sleep_or_abort(&hi_free[b], (uint32_t)(((st - 2) >> 1) & 1), &s_abort);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t s0 = tc_smem_addr(tiles + b * 3 * kGTile);
-                const uint32_t dhi = tmem + (uint32_t)(b * MN);
+        // ---- MMA issue (one elected lane of the converged warp): per stage, six
+        // split products per 16-point K step
+        const uint32_t idesc = umma_idesc_bf16(kGRows, MN);
+        const uint32_t el = tc_elect(), t0 = tc_uniform(tmem), tile0 = tc_uniform(tc_smem_addr(tiles));
+        for (int st = 0; st < nst && ok; ++st) {
+            const int b = st & 1;
+            ok = tc_mbar_sleep_or_abort(&conv_full[b], (uint32_t)((st >> 1) & 1), &s_abort);
+            // per-stage accumulator b was read back (stage st - 2)
+            if (ok && st >= 2) ok = tc_mbar_sleep_or_abort(&hi_free[b], (uint32_t)(((st - 2) >> 1) & 1), &s_abort);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t d0 = umma_desc_sw128(tile0 + (uint32_t)(b * 3 * kGTile));
+            const uint32_t dhi = t0 + (uint32_t)(b * MN), dx = t0 + (uint32_t)(2 * MN);
+            constexpr int pa[6] = {0, 0, 1, 0, 2, 1}, pb[6] = {0, 1, 0, 2, 0, 1};   // as c_pair_a, c_pair_b
 #pragma unroll
-                for (int kk = 0; kk < kGK / 16; ++kk) {
+            for (int kk = 0; kk < kGK / 16; ++kk) {
 #pragma unroll
-                    for (int p = 0; p < 6; ++p) {
-                        const uint64_t da = umma_desc_sw128(s0 + c_pair_a[p] * kGTile + kk * 32);
-                        const uint64_t db = umma_desc_sw128(s0 + c_pair_b[p] * kGTile + kk * 32);
-                        if (p == 0) umma_bf16(dhi, da, db, idesc, kk != 0);   // restarts every stage
-                        else umma_bf16(dcross, da, db, idesc, (st | kk | (p - 1)) != 0);
-                    }
+                for (int p = 0; p < 6; ++p) {
+                    const uint64_t da = d0 + (uint64_t)((pa[p] * kGTile + kk * 32) >> 4);
+                    const uint64_t db = d0 + (uint64_t)((pb[p] * kGTile + kk * 32) >> 4);
+                    if (p == 0) umma_bf16_el(dhi, da, db, idesc, kk != 0, el);   // restarts every stage
+                    else umma_bf16_el(dx, da, db, idesc, (st | kk | (p - 1)) != 0, el);
                 }
+            }
+            if (el) {
                 umma_commit(&mma_done[b]);
                 ++s_mma_issued;
             }
-            if (!ok) s_abort = 1;
+            __syncwarp();
         }
+        if (!ok && lane == 0) s_abort = 1;
         __syncwarp();
     } else {
         // ---- converters (warps 0-7); warps 0-3 also read the accumulators back

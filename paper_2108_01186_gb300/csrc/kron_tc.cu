@@ -78,9 +78,6 @@ constexpr uint32_t kTcColA = 256;                 // A operands: half h, split s
 constexpr int kTcMatElems = 64 * 64;              // one padded half-matrix
 constexpr int kTcOpElems = 12 * kTcMatElems;      // per operator: 2 directions x 2 halves x 3 splits
 
-__constant__ int c_tc_pa[6] = {0, 0, 1, 0, 2, 1};   // split of the data operand (A) of product p
-__constant__ int c_tc_pb[6] = {0, 1, 0, 2, 0, 1};   // split of the matrix operand (B)
-
 struct KronTcArgs {
     const BlkDesc* blk;
     int nblk;
@@ -191,7 +188,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
     __shared__ uint32_t tmem_base;
     __shared__ volatile int s_abort;
     __shared__ int s_tma_issued[2], s_mma_issued;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = (int)tc_uniform((uint32_t)tid >> 5), lane = tid & 31;
     const long long per_cta = (total + gridDim.x - 1) / gridDim.x;
     const long long it0 = (long long)blockIdx.x * per_cta;
     const long long it1 = it0 + per_cta < total ? it0 + per_cta : total;
@@ -226,55 +223,66 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
     const uint32_t tmem = tmem_base;
 
     if (warp == 0) {
-        // ---- control: copies and MMAs (lane 0) --------------------------------
-        if (lane == 0) {
-            TcBlk kc;
-            auto issue_copy = [&](const TcTile& t, int buf) {
-                tc_blk_load(kc, a.blk, t.b, a.axis);
-                const int nbox = (kc.n + 31) >> 5;
-                const int row0 = (int)((long long)t.o * kc.R + (long long)t.q * kTcRows);
-                unsigned char* dst = sR + buf * kTcRaw;
+        // ---- control: copies and MMAs (one elected lane of the converged warp) --
+        const uint32_t el = tc_elect();
+        TcBlk kc;
+        auto issue_copy = [&](const TcTile& t, int buf) {
+            tc_blk_load(kc, a.blk, t.b, a.axis);
+            const int nbox = (kc.n + 31) >> 5;
+            const int row0 = (int)((long long)t.o * kc.R + (long long)t.q * kTcRows);
+            unsigned char* dst = sR + buf * kTcRaw;
+            if (el) {
                 tc_mbar_expect_tx(&bar_tma[buf], (uint32_t)(nbox * kTcBox));
                 for (int bx = 0; bx < nbox; ++bx)
                     tc_tma_load_2d(dst + bx * kTcBox, a.maps + t.b, 32 * bx, row0, &bar_tma[buf]);
                 ++s_tma_issued[buf];
-            };
-            const uint32_t idesc = umma_idesc_bf16(kTcRows, kTcHalf);
-            const uint32_t b0 = tc_smem_addr(sB);
-            // copies run two tiles ahead: tile t (cur), t + 1 (t1, item n1), t + 2 (t2, item n2)
-            int bs = bsearch;
-            TcTile cur = first, t1{}, t2{};
-            long long n1 = tc_next(a, item0 + 1, it1, bs, t1);
-            long long n2 = n1 < it1 ? tc_next(a, n1 + 1, it1, bs, t2) : it1;
-            issue_copy(first, 0);
-            if (n1 < it1) issue_copy(t1, 1);
-            for (int t = 0;; ++t) {
-                // tile t's rows are read: the copy of tile t + 2 may land in their buffer
-                if (!tc_mbar_sleep_or_abort(&bar_raw[t & 1], (uint32_t)((t >> 1) & 1), &s_abort)) break;
-                if (n2 < it1) issue_copy(t2, t & 1);
-                bool ok = true;
-                for (int h = 0; h < 2 && ok; ++h) {
-                    ok = tc_mbar_sleep_or_abort(&bar_conv[h], (uint32_t)(t & 1), &s_abort);
-                    // the accumulators were read by the epilogue of tile t - 1
-                    if (ok && h == 0 && t >= 1)
-                        ok = tc_mbar_sleep_or_abort(&bar_empty, (uint32_t)((t - 1) & 1), &s_abort);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t dm = tmem + (uint32_t)(h * 128);
-                    const uint32_t am = tmem + kTcColA + (uint32_t)(h * 96);
-#pragma unroll 1
-                    for (int kk = 0; kk < 4; ++kk) {
+            }
+            __syncwarp();
+        };
+        const uint32_t idesc = umma_idesc_bf16(kTcRows, kTcHalf);
+        const uint32_t t0 = tc_uniform(tmem);
+        const uint64_t d0 = umma_desc_sw128(tc_uniform(tc_smem_addr(sB)));
+        constexpr int pa[6] = {0, 0, 1, 0, 2, 1};   // split of the data operand (A) of product p
+        constexpr int pb[6] = {0, 1, 0, 2, 0, 1};   // split of the matrix operand (B)
+        // copies run two tiles ahead: tile t (cur), t + 1 (t1, item n1), t + 2 (t2, item n2)
+        int bs = bsearch;
+        TcTile cur = first, t1{}, t2{};
+        long long n1 = tc_next(a, item0 + 1, it1, bs, t1);
+        long long n2 = n1 < it1 ? tc_next(a, n1 + 1, it1, bs, t2) : it1;
+        issue_copy(first, 0);
+        if (n1 < it1) issue_copy(t1, 1);
+        for (int t = 0;; ++t) {
+            // tile t's rows are read: the copy of tile t + 2 may land in their buffer
+            bool ok = tc_mbar_sleep_or_abort(&bar_raw[t & 1], (uint32_t)((t >> 1) & 1), &s_abort);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            if (n2 < it1) issue_copy(t2, t & 1);
 #pragma unroll
-                        for (int p = 0; p < 6; ++p) {
-                            const uint32_t ta = am + (uint32_t)(32 * c_tc_pa[p] + 8 * kk);
-                            const uint64_t db = umma_desc_sw128(b0 + (h * 3 + c_tc_pb[p]) * kTcBTile + kk * 32);
-                            if (p == 0) umma_bf16_ts(dm, ta, db, idesc, kk != 0);
-                            else umma_bf16_ts(dm + 64, ta, db, idesc, (kk | (p - 1)) != 0);
-                        }
-                    }
-                    umma_commit(&bar_half[h]);
-                }
+            for (int h = 0; h < 2; ++h) {
                 if (!ok) break;
+                ok = tc_mbar_sleep_or_abort(&bar_conv[h], (uint32_t)(t & 1), &s_abort);
+                // the accumulators were read by the epilogue of tile t - 1
+                if (ok && h == 0 && t >= 1)
+                    ok = tc_mbar_sleep_or_abort(&bar_empty, (uint32_t)((t - 1) & 1), &s_abort);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t dm = t0 + (uint32_t)(h * 128);
+                const uint32_t am = t0 + kTcColA + (uint32_t)(h * 96);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+#pragma unroll
+                    for (int p = 0; p < 6; ++p) {
+                        const uint32_t ta = am + (uint32_t)(32 * pa[p] + 8 * kk);
+                        const uint64_t db = d0 + (uint64_t)(((h * 3 + pb[p]) * kTcBTile + kk * 32) >> 4);
+                        if (p == 0) umma_bf16_ts_el(dm, ta, db, idesc, kk != 0, el);
+                        else umma_bf16_ts_el(dm + 64, ta, db, idesc, (kk | (p - 1)) != 0, el);
+                    }
+                }
+                if (el) umma_commit(&bar_half[h]);
+                __syncwarp();
+            }
+            if (!ok) break;
+            if (el) {
                 umma_commit(&bar_mma);
                 ++s_mma_issued;
                 if (a.flops) {
@@ -283,12 +291,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
                     const long long rows = B.G / n - (long long)cur.q * kTcRows;
                     atomicAdd(a.flops, 4.0 * (double)ns * ns * (double)(rows < kTcRows ? rows : kTcRows));
                 }
-                if (n1 >= it1) break;
-                cur = t1;
-                t1 = t2;
-                n1 = n2;
-                n2 = n1 < it1 ? tc_next(a, n1 + 1, it1, bs, t2) : it1;
             }
+            __syncwarp();
+            if (n1 >= it1) break;
+            cur = t1;
+            t1 = t2;
+            n1 = n2;
+            n2 = n1 < it1 ? tc_next(a, n1 + 1, it1, bs, t2) : it1;
         }
         __syncwarp();
     } else if (warp <= kTcConv / 32) {

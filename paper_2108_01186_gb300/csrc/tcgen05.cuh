@@ -87,13 +87,38 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
                  : "memory");
 }
 
-// D (tensor memory) (+)= A B^T with A in tensor memory (row i in lane i, two
-// bf16 K-values per 32-bit column) and B bf16 in shared memory
-__device__ __forceinline__ void umma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc, int acc) {
+// One lane of a converged warp (1 there, 0 in the others).  The MMAs below are
+// issued by a whole warp whose control flow and operands are warp-uniform,
+// predicated on this lane: the descriptors then live in uniform registers and
+// an M = 128, K = 16 MMA issues in N / 2 cycles (the tensor pipe's own rate:
+// 32 at N = 64, 64 at N = 128, measured).  Issued from a lane-0 branch, each
+// MMA moves its operands to uniform registers first and takes 86 cycles
+// whatever its N.
+__device__ __forceinline__ uint32_t tc_elect() {
+    uint32_t r;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r;
+}
+// a warp-uniform copy of v (lane 0's) that the compiler knows to be uniform
+__device__ __forceinline__ uint32_t tc_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+
+// D (tensor memory) (+)= A B^T issued by the elected lane of a converged warp:
+// both operands in shared memory, or A in tensor memory (row i in lane i, two
+// bf16 K-values per 32-bit column)
+__device__ __forceinline__ void umma_bf16_el(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, int acc,
+                                             uint32_t el) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc)
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+        "l"(da), "l"(db), "r"(idesc), "r"(acc), "r"(el)
+        : "memory");
+}
+__device__ __forceinline__ void umma_bf16_ts_el(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc, int acc,
+                                                uint32_t el) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc), "r"(el)
         : "memory");
 }
 
