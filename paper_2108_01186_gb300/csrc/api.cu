@@ -452,6 +452,16 @@ int flosic_create(flosic_ctx** out, const flosic_system* sys, int nsys, const fl
         for (int l = 0; l < M.nlev; ++l) {
             long long offl = 0, chl = 0, tl = 0;
             std::vector<int4> tiles;
+            const int depth = tile_depth(l == 0 ? kTileZ : kTileZc, l == 0 ? 4 : 1, c->num_sms, [&](int tz) {
+                long long n = 0;
+                for (int b = 0; b < c->nblk; ++b) {
+                    const BlkDesc& B = c->blk[b];
+                    if (l < nl[b])
+                        n += (long long)B.N * (((B.nx >> l) + kTileX - 1) / kTileX) *
+                             (((B.ny >> l) + kTileY - 1) / kTileY) * (((B.nz >> l) + tz - 1) / tz);
+                }
+                return n;
+            });
             for (int b = 0; b < c->nblk; ++b) {
                 const BlkDesc& B = c->blk[b];
                 LvlDesc D{};
@@ -478,7 +488,7 @@ int flosic_create(flosic_ctx** out, const flosic_system* sys, int nsys, const fl
                             if (m & (1 << k)) dd += (double)D.cl[k] - 2.0;
                         D.idd[m] = (float)(1.0 / dd);
                     }
-                    D.tz = (l == 0) ? kTileZ : kTileZc;
+                    D.tz = depth;
                     D.per = (l == 0) ? B.per : 0;
                     const int tx = (D.nx + kTileX - 1) / kTileX, ty = (D.ny + kTileY - 1) / kTileY,
                               tz = (D.nz + D.tz - 1) / D.tz;

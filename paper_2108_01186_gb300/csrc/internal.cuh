@@ -54,7 +54,19 @@ __host__ __device__ __forceinline__ int wrap_coord(int q, int n) { return q < 0 
 // One multigrid level of one spin block (level 0 = the fine grid).
 constexpr int kMaxLevels = 10;
 constexpr int kTileX = 32, kTileY = 16, kTileZ = 32;   // 3-D tiles of the sweeps (threads 32 x 8)
-constexpr int kTileZc = 4;   // tile z-depth on the coarse multigrid levels (enough CTAs to fill the GPU)
+constexpr int kTileZc = 4;   // largest tile z-depth on the coarse multigrid levels
+// A level's tile z-depth: the largest of max_tz, max_tz/2, .. min_tz that gives
+// the level (all blocks together, columns(tz) tiles) three tiles per SM, so
+// that small problems fill the GPU too.  A sweep re-reads 12 planes per tile,
+// which a problem this small finds in L2; at 40^3 x 5 the float64 stencil
+// sweep takes 220 us at depth 32 (60 tiles, each one serial z-march) and
+// 60 us at depth 4; larger problems keep the deepest tiles.
+template <class Tiles>
+inline int tile_depth(int max_tz, int min_tz, int num_sms, Tiles tiles) {
+    int tz = max_tz;
+    while (tz > min_tz && tiles(tz) < 3LL * num_sms) tz /= 2;
+    return tz;
+}
 constexpr int kCoarseSweeps = 40;      // damped-Jacobi sweeps on the coarsest level
 constexpr int kCoarseMax = 2000;       // largest coarsest level (points) kept in shared memory
 // planes of a tile staged with the 6-point x/y halo by the z-marching sweeps
@@ -74,7 +86,7 @@ struct LvlDesc {
     int tma;               // level 0: 1 if the stencil operands of this block are TMA-staged
     int utma;              // level 0: 1 if the refinement update's operands are TMA-staged
     int per;               // level 0: periodic directions (bit 0 x, 1 y, 2 z); 0 on coarse levels
-    int tz;                // z-depth of this level's tiles (kTileZ on level 0, kTileZc below)
+    int tz;                // z-depth of this level's tiles (see tile_depth)
     // Diagonal weight (units 1/h_l^2) of the 7-point operator at the last
     // point of each dimension, 2 elsewhere; differs from 2 on levels whose
     // parent had an even side (see multigrid.cu).  corr = any of them != 2.

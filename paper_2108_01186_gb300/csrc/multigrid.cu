@@ -181,28 +181,34 @@ __global__ void __launch_bounds__(256) k_mg_restrict(const BlkDesc* __restrict__
 #pragma unroll
         for (int k = 0; k < V; ++k) acc[k] = T(0);
         const int xf0 = 2 * X;
+        // the nine fine rows unrolled: their loads are independent and in flight
+        // together (rows past the grid count as zero)
+#pragma unroll
         for (int c = 0; c < 3; ++c) {
             const int zf = 2 * Z + c;
-            if (zf >= F.nz) continue;
             const T wc = (c == 1) ? T(0.5) : T(0.25);
+#pragma unroll
             for (int b = 0; b < 3; ++b) {
                 const int yf = 2 * Y + b;
-                if (yf >= F.ny) continue;
+                const bool ok = zf < F.nz && yf < F.ny;
                 const T w = wc * ((b == 1) ? T(0.5) : T(0.25));
-                const T* row = fb + zf * fz + yf * fy;
+                const T* row = fb + (ok ? zf * fz + yf * fy : 0);
                 T f[2 * V + 1];
                 if (n == V && fvec) {
-                    const VT a0 = *reinterpret_cast<const VT*>(row + xf0);
-                    const VT a1 = *reinterpret_cast<const VT*>(row + xf0 + V);
+                    VT a0{}, a1{};
+                    if (ok) {
+                        a0 = *reinterpret_cast<const VT*>(row + xf0);
+                        a1 = *reinterpret_cast<const VT*>(row + xf0 + V);
+                    }
 #pragma unroll
                     for (int k = 0; k < V; ++k) {
                         f[k] = reinterpret_cast<const T*>(&a0)[k];
                         f[V + k] = reinterpret_cast<const T*>(&a1)[k];
                     }
-                    f[2 * V] = (xf0 + 2 * V < F.nx) ? row[xf0 + 2 * V] : T(0);
+                    f[2 * V] = (ok && xf0 + 2 * V < F.nx) ? row[xf0 + 2 * V] : T(0);
                 } else {
 #pragma unroll
-                    for (int k = 0; k < 2 * V + 1; ++k) f[k] = (xf0 + k < F.nx) ? row[xf0 + k] : T(0);
+                    for (int k = 0; k < 2 * V + 1; ++k) f[k] = (ok && xf0 + k < F.nx) ? row[xf0 + k] : T(0);
                 }
 #pragma unroll
                 for (int k = 0; k < V; ++k)
