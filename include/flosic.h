@@ -125,13 +125,14 @@ typedef struct {
     int boundary;         /* FLOSIC_BC_ISOLATED (default), _PERIODIC, _SLAB */
     int kron_tensor_cores; /* KRON solver: 1 (default) runs the 1-D transforms
                              of every spin block whose sides are multiples of
-                             8 and at most 128 on the tensor cores (split
-                             bf16, float32 accumulation); 0 keeps them all on
-                             the CUDA cores (float32) */
+                             8 and at most 128, or all between 32 and 192, on
+                             the tensor cores (split bf16, float32
+                             accumulation); 0 keeps them all on the CUDA
+                             cores (float32) */
     int autotune;         /* KRON solver with kron_tensor_cores 1: 1 (default)
                              times, at context creation, one inner solve of
-                             each distinct block shape (nx, ny, nz, N) that
-                             qualifies for the tensor cores with the tensor-
+                             each distinct block shape (nx, ny, nz, N) with
+                             sides multiples of 8 up to 128 with the tensor-
                              core and with the CUDA-core transforms, and keeps
                              the faster per shape (flosic_block_paths reports
                              the choice); 0 takes the tensor cores wherever

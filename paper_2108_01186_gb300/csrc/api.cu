@@ -343,6 +343,25 @@ int flosic_create(flosic_ctx** out, const flosic_system* sys, int nsys, const fl
     }
     c->sgrid_elems = soff;
     sys_orb0[nsys] = orb;
+    // the Kronecker solver's float32 arrays: blocks that may take the tensor
+    // cores with padded sides, every block from a 16-byte boundary
+    {
+        const bool kron = o.solver == FLOSIC_SOLVER_KRON;
+        long long pe = 0;
+        for (BlkDesc& b : c->blk) {
+            const bool pad = kron && o.kron_tensor_cores && kron_tc_eligible(b);
+            const int n3[3] = {b.nx, b.ny, b.nz};
+            b.Gp = 1;
+            for (int d = 0; d < 3; ++d) {
+                b.p[d] = pad ? kron_pad(n3[d]) : n3[d];
+                b.Gp *= b.p[d];
+            }
+            for (int d = 0; d < 3; ++d) b.tpo[d] = kron_tc_tiles(b, d);
+            b.poff = kron ? (pe + 3) / 4 * 4 : b.off;
+            pe = b.poff + b.N * b.Gp;
+        }
+        c->pad_elems = pe;
+    }
     c->nblk = (int)c->blk.size();
     c->norb = orb;
     c->orb_elems = off;
@@ -414,7 +433,8 @@ int flosic_create(flosic_ctx** out, const flosic_system* sys, int nsys, const fl
     if (o.precision == FLOSIC_FP64) {
         A(&w.p64, off); A(&w.q64, off);
     } else {
-        A(&w.d32, off); A(&w.r32, off); A(&w.p32, off); A(&w.q32, off);
+        const long long pe = c->pad_elems;
+        A(&w.d32, pe); A(&w.r32, pe); A(&w.p32, pe); A(&w.q32, pe);
     }
     if (o.adjoint_mode == FLOSIC_ADJ_EXACT) A(&w.veff, off);
     if (uses_wbar(c)) A(&w.wbar, off);   // the only per-point adjoint input the mixed path needs

@@ -5,7 +5,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <map>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "../../include/flosic.h"
@@ -40,6 +42,14 @@ struct BlkDesc {
     long long kq[3];            // Kronecker solver: offsets of Q_d (then Q_d^T) in the matrix table
     long long kl[3];            // and of the eigenvalues of T_d
     long long kt[3];            // tensor-core transforms: offsets of the split bf16 matrices
+    long long klt[3];           // and of the eigenvalues of T_d in the padded mode order
+    // The Kronecker solver's float32 arrays (residual, correction, scratch) hold
+    // the block with every side padded to p (kron_pad) where it may take the
+    // tensor cores; p = n and, for the other solvers, poff = off otherwise.
+    int p[3];
+    int tpo[3];                 // tensor-core transforms: 128-row tiles per orbital of the pass along d
+    long long Gp;               // p[0] p[1] p[2]
+    long long poff;             // offset of orbital 0 in those arrays
     int tc;                     // 1: this block's transforms run on the tensor cores
     int gtma;                   // 1: the overlap Gram's psi tiles are staged by the copy engine
 };
@@ -186,6 +196,12 @@ namespace flosic {
 // Kronecker-product solver: transform matrices, eigenvalues and the launch
 // shape of its three passes (x, y, z lines).
 struct KronPlan {
+    // host eigen-decompositions per distinct operator (n, h, periodic): even and odd
+    // eigenvectors and eigenvalues, kept across the plans of one context
+    struct Eig {
+        std::vector<double> Vs, Va, ls, la;
+    };
+    std::map<std::tuple<int, double, int>, Eig> eig;
     float* mat = nullptr;          // per distinct 1-D operator: Q (n x n), then Q^T
     float* lam = nullptr;          // per distinct 1-D operator: eigenvalues (n)
     long long* items = nullptr;    // [3][nblk + 1] first tile of each block per pass (CUDA-core kernel)
@@ -195,12 +211,12 @@ struct KronPlan {
     int grid[3] = {0, 0, 0};
     int n_simt = 0, n_tc = 0;      // blocks on the CUDA-core and on the tensor-core transforms
     uint16_t* tc_mat = nullptr;    // per distinct operator of a tensor-core block: split bf16 matrices
-    long long* tc_items = nullptr; // [6][nblk + 1] first tile of each block per pass (tensor-core kernel)
+    long long* tc_items = nullptr; // [6 passes x 2 size classes][nblk + 1] first tile of each block (tensor-core kernel)
     std::vector<int> tc_force;     // [nblk] host: 0 = CUDA-core transforms even if eligible (autotuner)
     void* tc_maps = nullptr;       // [6][nblk] CUtensorMap of each pass's input rows
-    void* tc_omaps = nullptr;      // [6][nblk] CUtensorMap of each pass's output lines
-    long long tc_total[6] = {0, 0, 0, 0, 0, 0};
-    int tc_grid[6] = {0, 0, 0, 0, 0, 0};
+    long long tc_total[12] = {};
+    int tc_grid[12] = {};
+    int tc_full[12] = {};          // 1: every side of the pass and class fills the instance's half-lines
 };
 }  // namespace flosic
 
@@ -210,6 +226,7 @@ struct flosic_ctx {
     std::vector<flosic::BlkDesc> blk;       // host copy
     flosic::BlkDesc* d_blk = nullptr;       // device copy
     int nblk = 0, norb = 0;
+    long long pad_elems = 0;                // elements of the Kronecker solver's (padded) float32 arrays
     long long orb_elems = 0, vavg_elems = 0, mat_elems = 0, nchunk_total = 0;
     long long sgrid_elems = 0;   // sum over systems of the grid points (per-system fields)
     int kparts = 0;                         // K-splits of the grid contractions
@@ -325,15 +342,16 @@ cudaError_t setup_kron(flosic_ctx* c);
 void launch_kron_solve(flosic_ctx* c, const float* r, float* d, float* t1, float* t2, cudaStream_t s);
 // its transforms on the tensor cores (kron_tc.cu)
 bool kron_tc_eligible(const BlkDesc& B);
+bool kron_tc_tiled(const BlkDesc& B);   // every side a multiple of 8, at most 128 (no padding)
 // times the tensor-core and CUDA-core transforms per distinct eligible block
 // shape and re-plans the solver with the faster per shape (kron.cu)
 cudaError_t kron_autotune(flosic_ctx* c);
 void kron_tc_pack(int n, const std::vector<double>& Vs, const std::vector<double>& Va, std::vector<uint16_t>& out);
-size_t kron_tc_smem();
-const void* kron_tc_symbol();
+int kron_pad(int n);      // padded side of a line of n points
+int kron_tc_hp(int n);    // half-line size of the instance that takes sides of n points
+cudaError_t kron_tc_setup();
 bool kron_tc_map(void* encode_fn, CUtensorMap* map, const BlkDesc& B, int axis, const float* buf);
-bool kron_tc_map_out(void* encode_fn, CUtensorMap* map, const BlkDesc& B, int axis, float* buf);
-long long kron_tc_tiles(const BlkDesc& B, int axis);
+int kron_tc_tiles(const BlkDesc& B, int axis);   // per orbital
 void launch_kron_tc_pass(flosic_ctx* c, int step, float* out, cudaStream_t s);
 // Alternating Anderson-Richardson inner solver (mixed precision)
 template <class T>
@@ -563,6 +581,11 @@ __device__ __forceinline__ ff warp_sum(ff v) {
         v = ff_add(v, w);
     }
     return v;
+}
+
+// index of point (x, y, z) of orbital i of block B in the Kronecker solver's padded arrays
+__device__ __forceinline__ long long pad_index(const BlkDesc& B, int i, int x, int y, int z) {
+    return B.poff + (long long)i * B.Gp + ((long long)z * B.p[1] + y) * B.p[0] + x;
 }
 
 __device__ __forceinline__ int find_block(const BlkDesc* blk, int nblk, int orb) {

@@ -131,10 +131,11 @@ struct KronArgs {
 //   x: lines are grid rows (y, z), tile q = rows q*C .. q*C+C-1 (a contiguous run of C*nx values)
 //   y: lines are (x, z) columns at fixed z, tile q = (z, x-group)
 //   z: lines are xy points, tile q = xy points q*C .. q*C+C-1
+// (rows and xy points run over the padded sides of the arrays)
 __device__ __forceinline__ int pass_groups(const BlkDesc& B, int axis) {
-    if (axis == 0) return (B.ny * B.nz + kKronCols - 1) / kKronCols;
+    if (axis == 0) return (B.p[1] * B.nz + kKronCols - 1) / kKronCols;
     if (axis == 1) return B.nz * ((B.nx + kKronCols - 1) / kKronCols);
-    return (B.nx * B.ny + kKronCols - 1) / kKronCols;
+    return (B.p[0] * B.ny + kKronCols - 1) / kKronCols;
 }
 
 // Addressing of one tile: element (j, c) = position j along line c lies at
@@ -146,26 +147,26 @@ struct Tile {
 
 __device__ __forceinline__ Tile tile_of(const BlkDesc& B, int axis, int i_orb, int q) {
     Tile t;
-    const long long base = B.off + (long long)i_orb * B.G;
-    const long long sxy = (long long)B.nx * B.ny;
+    const long long base = B.poff + (long long)i_orb * B.Gp;
+    const long long px = B.p[0], sxy = px * B.p[1];
     t.q = q;
     if (axis == 0) {
-        t.cbase = base + (long long)q * kKronCols * B.nx;
-        t.cstride = B.nx;
+        t.cbase = base + (long long)q * kKronCols * px;
+        t.cstride = px;
         t.jstride = 1;
-        t.ncol = min(kKronCols, B.ny * B.nz - q * kKronCols);
+        t.ncol = min(kKronCols, B.p[1] * B.nz - q * kKronCols);
     } else if (axis == 1) {
         const int gx = (B.nx + kKronCols - 1) / kKronCols;
         const int zi = q / gx, xg = q - zi * gx;
         t.cbase = base + (long long)zi * sxy + (long long)xg * kKronCols;
         t.cstride = 1;
-        t.jstride = B.nx;
+        t.jstride = px;
         t.ncol = min(kKronCols, B.nx - xg * kKronCols);
     } else {
         t.cbase = base + (long long)q * kKronCols;
         t.cstride = 1;
         t.jstride = sxy;
-        t.ncol = (int)min((long long)kKronCols, sxy - (long long)q * kKronCols);
+        t.ncol = (int)min((long long)kKronCols, px * B.ny - (long long)q * kKronCols);
     }
     return t;
 }
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(2 * kKronMaxN) k_kron_pass(KronArgs a, long lo
         if (!a.inverse) {
             if (comp) {
                 if (a.scale) {   // forward z pass: column c is the xy mode (t % nx, t / nx)
-                    const long long sxy = (long long)B.nx * B.ny;
+                    const long long sxy = (long long)B.p[0] * B.ny;
                     const float* lx = a.lam + B.kl[0];
                     const float* ly = a.lam + B.kl[1];
                     const float* lz = a.lam + B.kl[2];
@@ -372,7 +373,7 @@ __global__ void __launch_bounds__(2 * kKronMaxN) k_kron_pass(KronArgs a, long lo
                     for (int v = 0; v < 4; ++v) {
                         const long long tt = (long long)t.q * kKronCols + c0 + v;
                         const int ti = (int)(tt < sxy ? tt : 0);
-                        const int yi = ti / B.nx, xi = ti - yi * B.nx;
+                        const int yi = ti / B.p[0], xi = ti - yi * B.p[0];
                         lxy[v] = lx[xi] + ly[yi];
                     }
 #pragma unroll
@@ -480,37 +481,40 @@ cudaError_t setup_kron_tc(flosic_ctx* c, const std::vector<uint16_t>& tcmat, int
     // the buffers of launch_kron_solve's passes as the refinement calls it
     // (r = r32, d = d32, scratch p32 and q32)
     const float* in_buf[6] = {c->ws.r32, c->ws.p32, c->ws.q32, c->ws.p32, c->ws.q32, c->ws.p32};
-    float* out_buf[6] = {c->ws.p32, c->ws.q32, c->ws.p32, c->ws.q32, c->ws.p32, c->ws.d32};
-    std::vector<CUtensorMap> maps(12 * (size_t)c->nblk);   // inputs, then outputs
-    std::vector<long long> items(6 * (size_t)(c->nblk + 1));
+    std::vector<CUtensorMap> maps(6 * (size_t)c->nblk);
+    std::vector<long long> items(12 * (size_t)(c->nblk + 1));
     std::memset(maps.data(), 0, sizeof(CUtensorMap) * maps.size());
     for (int st = 0; st < 6 && e == cudaSuccess; ++st) {
-        long long acc = 0;
-        for (int b = 0; b < c->nblk; ++b) {
-            const BlkDesc& B = c->blk[b];
-            items[(size_t)st * (c->nblk + 1) + b] = acc;
-            if (!B.tc) continue;
-            acc += kron_tc_tiles(B, st % 3);
-            if (!kron_tc_map(fn, &maps[(size_t)st * c->nblk + b], B, st % 3, in_buf[st]) ||
-                !kron_tc_map_out(fn, &maps[(size_t)(6 + st) * c->nblk + b], B, st % 3, out_buf[st]))
-                e = cudaErrorInvalidValue;
+        for (int cls = 0; cls < 2; ++cls) {   // sides up to 128, up to 192
+            const int k = 2 * st + cls;
+            long long acc = 0;
+            K.tc_full[k] = 1;
+            for (int b = 0; b < c->nblk; ++b) {
+                const BlkDesc& B = c->blk[b];
+                const int nd[3] = {B.nx, B.ny, B.nz};
+                items[(size_t)k * (c->nblk + 1) + b] = acc;
+                if (!B.tc || (kron_tc_hp(nd[st % 3]) > 64) != (cls == 1)) continue;
+                acc += (long long)B.N * B.tpo[st % 3];
+                if ((nd[st % 3] + 1) / 2 <= kron_tc_hp(nd[st % 3]) - 16) K.tc_full[k] = 0;
+                if (!kron_tc_map(fn, &maps[(size_t)st * c->nblk + b], B, st % 3, in_buf[st]))
+                    e = cudaErrorInvalidValue;
+            }
+            items[(size_t)k * (c->nblk + 1) + c->nblk] = acc;
+            K.tc_total[k] = acc;
+            K.tc_grid[k] = (int)(acc < sms ? (acc > 0 ? acc : 1) : sms);
         }
-        items[(size_t)st * (c->nblk + 1) + c->nblk] = acc;
-        K.tc_total[st] = acc;
-        K.tc_grid[st] = (int)(acc < sms ? (acc > 0 ? acc : 1) : sms);
     }
     void* dm = nullptr;
     if (e == cudaSuccess) e = cudaMalloc(&dm, sizeof(CUtensorMap) * maps.size());
     if (e == cudaSuccess) {
         c->allocations.push_back(dm);
         K.tc_maps = dm;
-        K.tc_omaps = reinterpret_cast<CUtensorMap*>(dm) + 6 * (size_t)c->nblk;
         e = cudaMemcpy(dm, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) e = ctx_alloc(c, &K.tc_items, items.size());
     if (e == cudaSuccess)
         e = cudaMemcpy(K.tc_items, items.data(), sizeof(long long) * items.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = ensure_dyn_smem(kron_tc_symbol(), kron_tc_smem());
+    if (e == cudaSuccess) e = kron_tc_setup();
     return e;
 }
 
@@ -520,7 +524,6 @@ cudaError_t setup_kron_tc(flosic_ctx* c, const std::vector<uint16_t>& tcmat, int
 // set to exactly zero), per-block offsets and the tile counts of the passes.
 cudaError_t setup_kron(flosic_ctx* c) {
     std::map<std::tuple<int, double, int>, std::pair<long long, long long>> seen;
-    std::map<std::tuple<int, double, int>, std::pair<std::vector<double>, std::vector<double>>> vecs;
     std::map<std::tuple<int, double, int>, long long> tc_seen;
     std::vector<float> mat, lam;
     std::vector<uint16_t> tcmat;
@@ -538,32 +541,38 @@ cudaError_t setup_kron(flosic_ctx* c) {
             const auto key = std::make_tuple(n, B.h, periodic);
             auto it = seen.find(key);
             if (it == seen.end()) {
-                const std::vector<double> T = axis_operator(n, B.h, periodic != 0);
                 const int ns = (n + 1) / 2, na = n / 2;
-                // even/odd basis: e_k = (d_k + d_{n-1-k}) / sqrt 2 (k < na), e_mid = d_mid;
-                // o_k = (d_k - d_{n-1-k}) / sqrt 2; T is persymmetric, so U^T T U is block diagonal
                 const double r2 = std::sqrt(0.5);
-                std::vector<double> Ts((size_t)ns * ns), Ta((size_t)na * na), Vs, Va;
-                // support of e_k / o_k: points k and n-1-k with weights (w, w) / (w, -w)
-                auto proj = [&](int k, int l, bool odd) {
-                    const int pk[2] = {k, n - 1 - k}, pl[2] = {l, n - 1 - l};
-                    const double wk = (!odd && k == n - 1 - k) ? 1.0 : r2;
-                    const double wl = (!odd && l == n - 1 - l) ? 1.0 : r2;
-                    const int mk = (pk[0] == pk[1]) ? 1 : 2, ml = (pl[0] == pl[1]) ? 1 : 2;
-                    double v = 0.0;
-                    for (int a = 0; a < mk; ++a)
-                        for (int b = 0; b < ml; ++b) {
-                            const double sa = (odd && a == 1) ? -1.0 : 1.0, sb = (odd && b == 1) ? -1.0 : 1.0;
-                            v += sa * wk * T[(size_t)pk[a] * n + pl[b]] * sb * wl;
-                        }
-                    return v;
-                };
-                for (int k = 0; k < ns; ++k)
-                    for (int l = 0; l < ns; ++l) Ts[(size_t)k * ns + l] = proj(k, l, false);
-                for (int k = 0; k < na; ++k)
-                    for (int l = 0; l < na; ++l) Ta[(size_t)k * na + l] = proj(k, l, true);
-                jacobi_eigen(ns, Ts, Vs);
-                if (na > 0) jacobi_eigen(na, Ta, Va);
+                KronPlan::Eig& E = K.eig[key];
+                if (E.ls.empty()) {
+                    const std::vector<double> T = axis_operator(n, B.h, periodic != 0);
+                    // even/odd basis: e_k = (d_k + d_{n-1-k}) / sqrt 2 (k < na), e_mid = d_mid;
+                    // o_k = (d_k - d_{n-1-k}) / sqrt 2; T is persymmetric, so U^T T U is block diagonal
+                    std::vector<double> Ts((size_t)ns * ns), Ta((size_t)na * na);
+                    // support of e_k / o_k: points k and n-1-k with weights (w, w) / (w, -w)
+                    auto proj = [&](int k, int l, bool odd) {
+                        const int pk[2] = {k, n - 1 - k}, pl[2] = {l, n - 1 - l};
+                        const double wk = (!odd && k == n - 1 - k) ? 1.0 : r2;
+                        const double wl = (!odd && l == n - 1 - l) ? 1.0 : r2;
+                        const int mk = (pk[0] == pk[1]) ? 1 : 2, ml = (pl[0] == pl[1]) ? 1 : 2;
+                        double v = 0.0;
+                        for (int a = 0; a < mk; ++a)
+                            for (int b = 0; b < ml; ++b) {
+                                const double sa = (odd && a == 1) ? -1.0 : 1.0, sb = (odd && b == 1) ? -1.0 : 1.0;
+                                v += sa * wk * T[(size_t)pk[a] * n + pl[b]] * sb * wl;
+                            }
+                        return v;
+                    };
+                    for (int k = 0; k < ns; ++k)
+                        for (int l = 0; l < ns; ++l) Ts[(size_t)k * ns + l] = proj(k, l, false);
+                    for (int k = 0; k < na; ++k)
+                        for (int l = 0; l < na; ++l) Ta[(size_t)k * na + l] = proj(k, l, true);
+                    jacobi_eigen(ns, Ts, E.Vs);
+                    if (na > 0) jacobi_eigen(na, Ta, E.Va);
+                    for (int k = 0; k < ns; ++k) E.ls.push_back(Ts[(size_t)k * ns + k]);
+                    for (int k = 0; k < na; ++k) E.la.push_back(Ta[(size_t)k * na + k]);
+                }
+                const std::vector<double>&Vs = E.Vs, &Va = E.Va;
                 // forward Fs[k][m] = Vs[k][m] fs_k (fs = 1/sqrt 2, 1/2 at the middle: s_mid = 2 v_mid),
                 // Fa = Va / sqrt 2; inverse in the kernel's transposed form Is[m][k] = Vs[k][m] gs_k
                 // (gs = 1/sqrt 2, 1 at the middle), Ia[m][k] = Va[k][m] / sqrt 2
@@ -587,23 +596,32 @@ cudaError_t setup_kron(flosic_ctx* c) {
                     }
                 int kmin = 0;   // the periodic constant mode is symmetric
                 for (int k = 0; k < ns; ++k) {
-                    lam.push_back((float)Ts[(size_t)k * ns + k]);
-                    if (std::fabs(Ts[(size_t)k * ns + k]) < std::fabs(Ts[(size_t)kmin * ns + kmin])) kmin = k;
+                    lam.push_back((float)E.ls[k]);
+                    if (std::fabs(E.ls[k]) < std::fabs(E.ls[kmin])) kmin = k;
                 }
-                for (int k = 0; k < na; ++k) lam.push_back((float)Ta[(size_t)k * na + k]);
+                for (int k = 0; k < na; ++k) lam.push_back((float)E.la[k]);
                 if (periodic) lam[lo + kmin] = 0.f;
+                // the same in the padded mode order of the tensor-core layouts (even modes
+                // at 0, odd at ns rounded up to 4; zeros between and 64 beyond the side)
+                {
+                    const int ns4 = (ns + 3) & ~3;
+                    const size_t l0 = lam.size();
+                    lam.resize(l0 + (size_t)kron_pad(n) + 64, 0.f);
+                    for (int k = 0; k < ns; ++k) lam[l0 + k] = lam[lo + k];
+                    for (int k = 0; k < na; ++k) lam[l0 + ns4 + k] = lam[lo + ns + k];
+                }
                 it = seen.emplace(key, std::make_pair(qo, lo)).first;
-                vecs.emplace(key, std::make_pair(std::move(Vs), std::move(Va)));
             }
             B.kq[d] = it->second.first;
             B.kl[d] = it->second.second;
+            B.klt[d] = B.kl[d] + n;
             B.kt[d] = 0;
             if (B.tc) {
                 auto jt = tc_seen.find(key);
                 if (jt == tc_seen.end()) {
-                    const auto& V = vecs.at(key);
+                    const KronPlan::Eig& V = K.eig.at(key);
                     const long long to = (long long)tcmat.size();
-                    kron_tc_pack(n, V.first, V.second, tcmat);
+                    kron_tc_pack(n, V.Vs, V.Va, tcmat);
                     jt = tc_seen.emplace(key, to).first;
                 }
                 B.kt[d] = jt->second;
@@ -624,9 +642,9 @@ cudaError_t setup_kron(flosic_ctx* c) {
             const BlkDesc& B = c->blk[b];
             items[(size_t)d * (c->nblk + 1) + b] = acc;
             long long g;
-            if (d == 0) g = (B.ny * (long long)B.nz + kKronCols - 1) / kKronCols;
+            if (d == 0) g = (B.p[1] * (long long)B.nz + kKronCols - 1) / kKronCols;
             else if (d == 1) g = (long long)B.nz * ((B.nx + kKronCols - 1) / kKronCols);
-            else g = ((long long)B.nx * B.ny + kKronCols - 1) / kKronCols;
+            else g = ((long long)B.p[0] * B.ny + kKronCols - 1) / kKronCols;
             if (!B.tc) acc += g * B.N;   // tensor-core blocks take no tiles of this kernel
             const int n = d == 0 ? B.nx : (d == 1 ? B.ny : B.nz);
             nmax = n > nmax ? n : nmax;
@@ -660,7 +678,8 @@ cudaError_t setup_kron(flosic_ctx* c) {
 }
 
 // Autotuner of the transforms: per distinct shape (nx, ny, nz, N, periodic
-// sides) of the blocks that qualify for the tensor cores, one inner solve of
+// sides) of the blocks whose sides are multiples of 8 up to 128 (the padded
+// shapes always take the tensor cores), one inner solve of
 // one block of that shape is timed (CUDA events, after a warm-up solve, three
 // solves averaged, zero input: the transforms' cost does not depend on the
 // values) with every qualifying block on the tensor cores and again with
@@ -671,7 +690,7 @@ cudaError_t kron_autotune(flosic_ctx* c) {
     std::map<std::array<long long, 5>, std::vector<int>> groups;
     for (int b = 0; b < c->nblk; ++b) {
         const BlkDesc& B = c->blk[b];
-        if (kron_tc_eligible(B)) groups[{B.nx, B.ny, B.nz, B.N, B.per}].push_back(b);
+        if (kron_tc_tiled(B)) groups[{B.nx, B.ny, B.nz, B.N, B.per}].push_back(b);
     }
     if (groups.empty()) return cudaSuccess;
     cudaStream_t s = nullptr;
@@ -681,7 +700,7 @@ cudaError_t kron_autotune(flosic_ctx* c) {
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     if (e == cudaSuccess) e = cudaMalloc(&dflags, sizeof(int) * (size_t)c->norb * groups.size());
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws.r32, 0, sizeof(float) * (size_t)c->orb_elems, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws.r32, 0, sizeof(float) * (size_t)c->pad_elems, s);
     // per group: only the first block's orbitals active
     std::vector<int> hflags((size_t)c->norb * groups.size(), 0);
     {

@@ -76,8 +76,11 @@ __global__ void __launch_bounds__(256) k_ff_init(const BlkDesc* __restrict__ blk
     const TilePos P = tile_pos(blk, L, tiles, orb_blk, blockIdx.x);
     if (!st.oactive[P.o]) return;
     const LvlDesc& D = L[P.b];
+    const BlkDesc& B = blk[P.b];
+    const int io = P.o - B.orb0;
     float bb = 0.f;
-    tile_elementwise<float>(D, P, [&](long long g, int n) {
+    tile_rows<float>(D, P, [&](int px, int py, int pz, long long g, int n) {
+        const long long q = pad_index(B, io, px, py, pz);   // in r32 (and p32, d32)
         if (n == 4) {   // aligned group of four points: 16-byte accesses
             const float4 b01 = *reinterpret_cast<const float4*>(b + g);       // pairs g, g+1
             const float4 b23 = *reinterpret_cast<const float4*>(b + g + 2);   // pairs g+2, g+3
@@ -94,10 +97,10 @@ __global__ void __launch_bounds__(256) k_ff_init(const BlkDesc* __restrict__ blk
                 if (!keep_zero) {
                     *reinterpret_cast<float4*>(x + g) = z4;
                     *reinterpret_cast<float4*>(x + g + 2) = z4;
-                    *reinterpret_cast<float4*>(d32 + g) = z4;
+                    *reinterpret_cast<float4*>(d32 + q) = z4;
                 }
-                *reinterpret_cast<float4*>(r32 + g) = bh;
-                if (p32) *reinterpret_cast<float4*>(p32 + g) = bh;
+                *reinterpret_cast<float4*>(r32 + q) = bh;
+                if (p32) *reinterpret_cast<float4*>(p32 + q) = bh;
             }
             return;
         }
@@ -109,10 +112,10 @@ __global__ void __launch_bounds__(256) k_ff_init(const BlkDesc* __restrict__ blk
             } else {
                 if (!keep_zero) {
                     x[g + k] = make_float2(0.f, 0.f);
-                    d32[g + k] = 0.f;
+                    d32[q + k] = 0.f;
                 }
-                r32[g + k] = bh;
-                if (p32) p32[g + k] = bh;
+                r32[q + k] = bh;
+                if (p32) p32[q + k] = bh;
             }
         }
     });
@@ -143,6 +146,8 @@ __global__ void __launch_bounds__(256) k_residual12_ff(const BlkDesc* __restrict
     if (!st.oactive[P.o]) return;
     const LvlDesc& D = L[P.b];
     const ff ih2 = to_ff(d2ff(1.0 / (D.h * D.h)));   // once per CTA
+    const BlkDesc& B = blk[P.b];
+    const bool padded = B.Gp != B.G;
     float rrf = 0.f;
     ff_sweep12<true>(
         D, P, [&](long long g) { return x[g]; },
@@ -151,9 +156,14 @@ __global__ void __launch_bounds__(256) k_residual12_ff(const BlkDesc* __restrict
             const ff r = ff_add(to_ff(b[g]), ff_mul(acc, ih2));
             const float rv = r.h;
             if (store_r) b[g] = make_float2(r.h, r.l);
-            r32[g] = rv;
-            d32[g] = 0.f;
-            if (p32) p32[g] = rv;
+            long long q = g - P.base + B.poff + (long long)(P.o - B.orb0) * B.Gp;   // in r32, p32, d32
+            if (padded) {
+                const unsigned i = (unsigned)(g - P.base), row = i / (unsigned)D.nx, z = row / (unsigned)D.ny;
+                q = pad_index(B, P.o - B.orb0, (int)(i - row * D.nx), (int)(row - z * D.ny), (int)z);
+            }
+            r32[q] = rv;
+            d32[q] = 0.f;
+            if (p32) p32[q] = rv;
             rrf += rv * rv;
         },
         plane);
@@ -266,8 +276,12 @@ __global__ void __launch_bounds__(256) k_dmax(const BlkDesc* __restrict__ blk, c
     const TilePos P = tile_pos(blk, L, tiles, orb_blk, blockIdx.x);
     if (!st.oactive[P.o]) return;
     const LvlDesc& D = L[P.b];
+    const BlkDesc& B = blk[P.b];
+    if (B.tc) return;   // recorded by the tensor-core transforms
+    const int io = P.o - B.orb0;
     float m = 0.f;
-    tile_elementwise<float>(D, P, [&](long long g, int n) {
+    tile_rows<float>(D, P, [&](int px, int py, int pz, long long, int n) {
+        const long long g = pad_index(B, io, px, py, pz);
         if (n == 4) {
             const float4 v = *reinterpret_cast<const float4*>(d32 + g);
             m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
@@ -322,6 +336,11 @@ __global__ void __launch_bounds__(256, 2) k_update12_ix(const BlkDesc* __restric
     const int gy0 = P.y0 + ty, gy1 = P.y0 + ty + kTileY / 2;
     const bool in0 = gx < D.nx && gy0 < D.ny, in1 = gx < D.nx && gy1 < D.ny;
     const long long c0 = gy0 * sy + gx, c1 = gy1 * sy + gx;
+    // d and r32 hold the block with padded sides: plane and row strides, the orbital's offset
+    const BlkDesc& B = blk[P.b];
+    const int dpx = B.p[0];
+    const long long dsz = (long long)dpx * B.p[1], db = B.poff + (long long)(P.o - B.orb0) * B.Gp;
+    const long long e0 = (long long)gy0 * dpx + gx, e1 = (long long)gy1 * dpx + gx;
     int soff[kSlots];   // in-plane offsets of this thread's staged points (-1: outside)
 #pragma unroll
     for (int j = 0; j < kSlots; ++j) {
@@ -332,7 +351,7 @@ __global__ void __launch_bounds__(256, 2) k_update12_ix(const BlkDesc* __restric
             int px = P.x0 - kHalf + xx, py = P.y0 - kHalf + yy;
             if (D.per & 1) px = wrap_coord(px, D.nx);
             if (D.per & 2) py = wrap_coord(py, D.ny);
-            if (px >= 0 && px < D.nx && py >= 0 && py < D.ny) soff[j] = py * D.nx + px;
+            if (px >= 0 && px < D.nx && py >= 0 && py < D.ny) soff[j] = py * dpx + px;
         }
     }
     IxPt q0[2 * kHalf + 1], q1[2 * kHalf + 1];
@@ -342,12 +361,12 @@ __global__ void __launch_bounds__(256, 2) k_update12_ix(const BlkDesc* __restric
         int zz = P.z0 - kHalf + j;
         if (perz) zz = wrap_coord(zz, D.nz);
         const bool okz = zz >= 0 && zz < D.nz;
-        q0[j] = ix_split((in0 && okz) ? d32[P.base + zz * sz + c0] : 0.f, s);
-        q1[j] = ix_split((in1 && okz) ? d32[P.base + zz * sz + c1] : 0.f, s);
+        q0[j] = ix_split((in0 && okz) ? d32[db + zz * dsz + e0] : 0.f, s);
+        q1[j] = ix_split((in1 && okz) ? d32[db + zz * dsz + e1] : 0.f, s);
     }
     float pre[kSlots];
 #pragma unroll
-    for (int j = 0; j < kSlots; ++j) pre[j] = (soff[j] >= 0) ? d32[P.base + P.z0 * sz + soff[j]] : 0.f;
+    for (int j = 0; j < kSlots; ++j) pre[j] = (soff[j] >= 0) ? d32[db + P.z0 * dsz + soff[j]] : 0.f;
     // r and x of this thread's two points, one plane ahead of their use
     constexpr bool xz = kXZ;
     const float2 f0 = make_float2(0.f, 0.f);
@@ -371,15 +390,15 @@ __global__ void __launch_bounds__(256, 2) k_update12_ix(const BlkDesc* __restric
         {
             int zz = z + kHalf;
             if (perz) zz = wrap_coord(zz, D.nz);
-            q0[2 * kHalf] = ix_split((in0 && zz < D.nz) ? d32[P.base + zz * sz + c0] : 0.f, s);
-            q1[2 * kHalf] = ix_split((in1 && zz < D.nz) ? d32[P.base + zz * sz + c1] : 0.f, s);
+            q0[2 * kHalf] = ix_split((in0 && zz < D.nz) ? d32[db + zz * dsz + e0] : 0.f, s);
+            q1[2 * kHalf] = ix_split((in1 && zz < D.nz) ? d32[db + zz * dsz + e1] : 0.f, s);
         }
         __syncthreads();
         float4 nx0 = rx0, nx1 = rx1;
         if (z + 1 < P.z1) {
             const long long pz = P.base + (z + 1) * sz;
 #pragma unroll
-            for (int j = 0; j < kSlots; ++j) pre[j] = (soff[j] >= 0) ? d32[pz + soff[j]] : 0.f;
+            for (int j = 0; j < kSlots; ++j) pre[j] = (soff[j] >= 0) ? d32[db + (z + 1) * dsz + soff[j]] : 0.f;
             if (in0) {
                 const float2 rv = r[pz + c0], xv = xz ? f0 : x[pz + c0];
                 nx0 = make_float4(rv.x, rv.y, xv.x, xv.y);
@@ -419,7 +438,7 @@ __global__ void __launch_bounds__(256, 2) k_update12_ix(const BlkDesc* __restric
                 const ff xn = ff_quick(xs.h, xs.l + rx.w);
                 r[g] = make_float2(rn.h, rn.l);
                 x[g] = make_float2(xn.h, xn.l);
-                r32[g] = rn.h;
+                r32[db + z * dsz + (k == 0 ? e0 : e1)] = rn.h;
                 rrf += rn.h * rn.h;
             }
         }
@@ -514,9 +533,13 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
     __syncthreads();
     const int tx = threadIdx.x, ty = threadIdx.y;   // 16 x 16
     const int gx = P.x0 + 2 * tx, gy = P.y0 + ty;
-    const bool in = gx < D.nx && gy < D.ny;           // nx is a multiple of 4: gx + 1 < nx as well
+    const bool in = gx < D.nx && gy < D.ny;           // nx is even: gx + 1 < nx as well
     const long long sy = D.nx, sz = (long long)D.nx * D.ny;
     const long long col = gy * sy + gx;
+    // d and r32 hold the block with padded sides
+    const BlkDesc& B = blk[P.b];
+    const long long dsz = (long long)B.p[0] * B.p[1];
+    const long long dcol = B.poff + (long long)oi * B.Gp + (long long)gy * B.p[0] + gx;
     // z-windows of the two points as rings of 13 registers: plane z - 6 + j of
     // step k sits in slot (k + j) mod 13, so nothing moves between planes (the
     // z-loop is unrolled by 13 to make every slot index a constant)
@@ -526,7 +549,7 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
     for (int j = 0; j < 2 * kHalf; ++j) {
         const int zz = P.z0 - kHalf + j;
         float2 v = make_float2(0.f, 0.f);
-        if (in && zz >= 0 && zz < D.nz) v = *reinterpret_cast<const float2*>(d32 + P.base + zz * sz + col);
+        if (in && zz >= 0 && zz < D.nz) v = *reinterpret_cast<const float2*>(d32 + zz * dsz + dcol);
         q0[j] = ix_split_w(v.x, sc);
         q1[j] = ix_split_w(v.y, sc);
     }
@@ -603,7 +626,7 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
                 }
                 *reinterpret_cast<float4*>(r + g) = make_float4(rn[0].h, rn[0].l, rn[1].h, rn[1].l);
                 *reinterpret_cast<float4*>(x + g) = make_float4(xn[0].h, xn[0].l, xn[1].h, xn[1].l);
-                *reinterpret_cast<float2*>(r32 + g) = make_float2(rn[0].h, rn[1].h);
+                *reinterpret_cast<float2*>(r32 + (P.z0 + k) * dsz + dcol) = make_float2(rn[0].h, rn[1].h);
             }
         }
     }
@@ -637,16 +660,16 @@ int setup_update_maps(flosic_ctx* c) {
     for (int b = 0; b < c->nblk; ++b) {
         const BlkDesc& B = c->blk[b];
         L0[b].utma = 0;
-        if (B.nx % 4 != 0 || B.off % 4 != 0 || B.per != 0) continue;
+        if (B.p[0] % 4 != 0 || B.poff % 4 != 0 || B.nx % 2 != 0 || B.off % 2 != 0 || B.per != 0) continue;
         const cuuint64_t dims[4] = {(cuuint64_t)B.nx, (cuuint64_t)B.ny, (cuuint64_t)B.nz, (cuuint64_t)B.N};
-        const cuuint64_t strides[3] = {(cuuint64_t)B.nx * 4, (cuuint64_t)B.nx * B.ny * 4, (cuuint64_t)B.G * 4};
+        const cuuint64_t strides[3] = {(cuuint64_t)B.p[0] * 4, (cuuint64_t)B.p[0] * B.p[1] * 4, (cuuint64_t)B.Gp * 4};
         const cuuint64_t dims2[4] = {2 * (cuuint64_t)B.nx, (cuuint64_t)B.ny, (cuuint64_t)B.nz, (cuuint64_t)B.N};
         const cuuint64_t strides2[3] = {(cuuint64_t)B.nx * 8, (cuuint64_t)B.nx * B.ny * 8, (cuuint64_t)B.G * 8};
         const cuuint32_t box_halo[4] = {(cuuint32_t)kUX, (cuuint32_t)kUY, 1, 1};
         const cuuint32_t box_ctr[4] = {(cuuint32_t)kTileX, (cuuint32_t)kTileY, 1, 1};
         const cuuint32_t box_pair[4] = {2 * (cuuint32_t)kTileX, (cuuint32_t)kTileY, 1, 1};
         const cuuint32_t estr[4] = {1, 1, 1, 1};
-        float* d = c->ws.d32 + B.off;
+        float* d = c->ws.d32 + B.poff;
         float* rb = reinterpret_cast<float*>(c->ws.b64 + B.off);
         float* xb = reinterpret_cast<float*>(c->ws.r64 + B.off);
         bool ok = true;

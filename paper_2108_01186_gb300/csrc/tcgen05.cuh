@@ -67,6 +67,17 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
     return d;
 }
 
+// The same with a 64-byte swizzle: rows of 64 bytes (32 bf16), 8-row groups
+// 512 bytes apart, 16-byte piece c of row m at c ^ ((m >> 1) & 3).
+__device__ __forceinline__ uint64_t umma_desc_sw64(uint32_t saddr) {
+    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(512 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;                  // 64-byte swizzle
+    return d;
+}
+
 // Instruction descriptor of kind::f16: bf16 A and B (K-major), float32 D.
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
@@ -99,8 +110,9 @@ __device__ __forceinline__ uint32_t tc_elect() {
     asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
     return r;
 }
-// a warp-uniform copy of v (lane 0's) that the compiler knows to be uniform
-__device__ __forceinline__ uint32_t tc_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+// A warp-uniform value v in a form that the compiler knows to be uniform (the
+// reduction's result is a uniform register; a shuffle's is not).
+__device__ __forceinline__ uint32_t tc_uniform(uint32_t v) { return __reduce_or_sync(0xffffffffu, v); }
 
 // D (tensor memory) (+)= A B^T issued by the elected lane of a converged warp:
 // both operands in shared memory, or A in tensor memory (row i in lane i, two
@@ -141,6 +153,8 @@ __device__ __forceinline__ void tc_tma_store_2d(const CUtensorMap* map, int c0, 
 __device__ __forceinline__ void tc_bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // at most one committed bulk group still reads shared memory
 __device__ __forceinline__ void tc_bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
+// no committed bulk group still reads shared memory
+__device__ __forceinline__ void tc_bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // every committed bulk group has completed
 __device__ __forceinline__ void tc_bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
