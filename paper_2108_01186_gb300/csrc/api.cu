@@ -467,6 +467,22 @@ int flosic_create(flosic_ctx** out, const flosic_system* sys, int nsys, const fl
             for (int b = 0; b < c->nblk; ++b) { nl[b] = 1; coarsest[b] = 0; }
         }
         const size_t tsz = (o.precision == FLOSIC_FP64) ? sizeof(double) : sizeof(float);
+        // the levels that k_mg_coarse takes: from the first one of at most mg_fuse_max
+        // points that fits in shared memory with those below it (always the coarsest)
+        std::vector<int> fused = coarsest;
+        for (int b = 0; b < c->nblk && M.enabled; ++b) {
+            const BlkDesc& B = c->blk[b];
+            auto bytes = [&](int l) {
+                return (size_t)mg_coarse_elems(B.nx >> l, B.ny >> l, B.nz >> l, nl[b] - l) * tsz;
+            };
+            while (fused[b] > 0) {
+                const int l = fused[b] - 1;
+                if ((long long)(B.nx >> l) * (B.ny >> l) * (B.nz >> l) > mg_fuse_max(tsz) || bytes(l) > kMgSmemMax) break;
+                fused[b] = l;
+            }
+            M.fused_max = std::max(M.fused_max, fused[b]);
+            M.coarse_smem = std::max(M.coarse_smem, bytes(fused[b]));
+        }
         // last-point diagonal weights per block and dimension, level by level
         std::vector<std::array<double, 3>> cl(c->nblk, std::array<double, 3>{2.0, 2.0, 2.0});
         for (int l = 0; l < M.nlev; ++l) {
@@ -493,7 +509,7 @@ int flosic_create(flosic_ctx** out, const flosic_system* sys, int nsys, const fl
                     D.h = B.h * (double)(1 << l);
                     D.G = (long long)D.nx * D.ny * D.nz;
                     D.nchunk = (int)((D.G + kChunk - 1) / kChunk);
-                    D.coarsest = (l == nl[b] - 1) ? 1 : 0;
+                    D.fused = (l >= fused[b]) ? 1 : 0;
                     const int sides[3] = {D.nx, D.ny, D.nz};
                     D.corr = 0;
                     for (int k = 0; k < 3; ++k) {
@@ -542,6 +558,10 @@ int flosic_create(flosic_ctx** out, const flosic_system* sys, int nsys, const fl
         A(&M.d_coarsest_level, c->nblk);
         if (e == cudaSuccess)
             e = cudaMemcpy(M.d_coarsest_level, coarsest.data(), sizeof(int) * c->nblk, cudaMemcpyHostToDevice);
+        A(&M.d_fused_level, c->nblk);
+        if (e == cudaSuccess)
+            e = cudaMemcpy(M.d_fused_level, fused.data(), sizeof(int) * c->nblk, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess && M.enabled) e = setup_mg_coarse(c);
         if (o.precision == FLOSIC_FP64) {
             if (M.enabled) { A(&w.z64, off); A(&w.p64b, off); }
         } else if (M.enabled || o.solver == FLOSIC_SOLVER_AAR) {

@@ -79,13 +79,20 @@ inline int tile_depth(int max_tz, int min_tz, int num_sms, Tiles tiles) {
 }
 constexpr int kCoarseSweeps = 40;      // damped-Jacobi sweeps on the coarsest level
 constexpr int kCoarseMax = 2000;       // largest coarsest level (points) kept in shared memory
+// Levels that the V-cycle runs in one launch, a CTA per orbital (k_mg_coarse):
+// in float32 as many as fit in shared memory (24^3 points and those below); in
+// float64 levels of up to 2000 points, where a CTA's float64 pipe (1.7 FMA per
+// cycle) takes less than the 30 us of the level's four launches.
+constexpr size_t kMgSmemMax = 200 * 1024;
+constexpr long long mg_fuse_max(size_t elem) { return elem == sizeof(float) ? 14000 : 2000; }
+long long mg_coarse_elems(int nx, int ny, int nz, int nlev);
 // planes of a tile staged with the 6-point x/y halo by the z-marching sweeps
 constexpr int kPX = kTileX + 2 * kHalf;   // staged plane width
 constexpr int kPY = kTileY + 2 * kHalf;   // staged plane height
 constexpr int kSlots = (kPX * kPY + kTileX * (kTileY / 2) - 1) / (kTileX * (kTileY / 2));   // per thread
 struct LvlDesc {
     int nx, ny, nz;
-    int coarsest;          // 1 if this is the block's last level
+    int fused;             // 1 if this level runs in shared memory with those below it (k_mg_coarse)
     double h;              // 2^l h
     long long G;           // points (0: the block has no such level)
     long long off;         // offset of orbital 0 in this level's arrays
@@ -115,6 +122,7 @@ struct MgPtrs {
     T* t[kMaxLevels];      // scratch (level 0: the CG q buffer, idle during the V-cycle)
     const LvlDesc* lvl[kMaxLevels];
     const int* coarsest_level;   // [nblk]
+    const int* fused_level;      // [nblk] first level of k_mg_coarse
 };
 
 // Per-orbital state of the batched conjugate-gradient solver.
@@ -182,6 +190,9 @@ struct Multigrid {
     long long nchunk[kMaxLevels] = {};         // chunks per level (all orbitals)
     long long elems[kMaxLevels] = {};          // elements per level (all orbitals)
     int* d_coarsest_level = nullptr;           // [nblk]
+    int* d_fused_level = nullptr;              // [nblk]
+    int fused_max = 0;                         // the largest of them
+    size_t coarse_smem = 0;                    // shared memory of k_mg_coarse
     int4* d_tiles[kMaxLevels] = {};            // tile -> (orbital, x0, y0, z0) per level
     long long ntiles[kMaxLevels] = {};
     long long coarsest_max = 0;
@@ -378,6 +389,7 @@ size_t apply12_tma_smem(size_t elem);
 const void* apply12_tma_symbol(bool f32);
 void launch_residual12(flosic_ctx* c, const double* b, const double* x, double* r, double tol2, int max_iter,
                        int* flag, int* counter, int want_bb, cudaStream_t s);
+cudaError_t setup_mg_coarse(const flosic_ctx* c);
 cudaError_t upload_ff_weights();
 int setup_update_maps(flosic_ctx* c);   // refinement update's tensor maps (refine.cu); blocks on that path
 // mixed precision: float-float refinement around the float32 inner solves

@@ -19,13 +19,13 @@
 // loses most of its strength on grids such as 128^3.  Restriction is full
 // weighting (1/4, 1/2, 1/4 per direction) = (1/8) P^T with P trilinear
 // interpolation.  Smoother: one damped-Jacobi sweep before and after
-// (omega = 0.8); coarsest level: 40 damped-Jacobi sweeps from zero in shared
-// memory.  Every piece is symmetric and the smoother converges in the A2
+// (omega = 0.8); coarsest level: 40 damped-Jacobi sweeps from zero.  Every piece is symmetric and the smoother converges in the A2
 // norm, so the V-cycle is a symmetric positive definite operator.
 //
 // Kernels work on per-level tables of 3-D tiles (one CTA per 32 x 16 x 32
 // tile of one orbital) so that all orbitals of all systems run in one launch
-// per level.
+// per level; the levels small enough for shared memory run in one launch
+// together (k_mg_coarse).
 #include "internal.cuh"
 
 namespace flosic {
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(256) k_mg_resid_smooth(const BlkDesc* __restri
     constexpr int V = Vec<T>::n;
     const TilePos P = tile_pos(blk, L, tiles, orb_blk, blockIdx.x);
     const LvlDesc& D = L[P.b];
-    if (!active[P.o] || D.coarsest) return;
+    if (!active[P.o] || D.fused) return;
     const long long sy = D.nx, sz = (long long)D.nx * D.ny;
     tile_rows<T>(D, P, [&](int x, int y, int z, long long g, int n) {
         if (D.corr && (x + n >= D.nx - 1 || y >= D.ny - 2 || z >= D.nz - 2)) {
@@ -169,9 +169,9 @@ __global__ void __launch_bounds__(256) k_mg_restrict(const BlkDesc* __restrict__
     constexpr int V = Vec<T>::n;
     using VT = typename Vec<T>::type;
     const TilePos P = tile_pos(blk, Lc, tiles_c, orb_blk, blockIdx.x);
-    if (!active[P.o]) return;
     const LvlDesc& C = Lc[P.b];
     const LvlDesc& F = Lf[P.b];
+    if (!active[P.o] || F.fused) return;
     const long long fbase = F.off + (long long)(P.o - blk[P.b].orb0) * F.G;
     const T* fb = sf + fbase;
     const long long fy = F.nx, fz = (long long)F.nx * F.ny;
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(256) k_mg_prolong(const BlkDesc* __restrict__ 
                                                     T* __restrict__ t, T omega) {
     const TilePos P = tile_pos(blk, Lf, tiles_f, orb_blk, blockIdx.x);
     const LvlDesc& F = Lf[P.b];
-    if (!active[P.o] || F.coarsest) return;
+    if (!active[P.o] || F.fused) return;
     const LvlDesc& C = Lc[P.b];
     const T* eb = ec + C.off + (long long)(P.o - blk[P.b].orb0) * C.G;
     const T oh2 = omega * T(F.h * F.h);
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(256) k_mg_postsmooth(const BlkDesc* __restrict
     __shared__ double scratch[32];
     const TilePos P = tile_pos(blk, L, tiles, orb_blk, blockIdx.x);
     const LvlDesc& D = L[P.b];
-    if (!active[P.o] || D.coarsest) return;
+    if (!active[P.o] || D.fused) return;
     const T h2 = T(D.h * D.h);
     T rz = T(0);   // per-thread partial in the working precision; tile sums in float64
     tile_rows<T>(D, P, [&](int x, int y, int z, long long g, int n) {
@@ -453,53 +453,202 @@ __global__ void __launch_bounds__(256) k_mg_postsmooth(const BlkDesc* __restrict
     }
 }
 
-// Coarsest level of each block: damped Jacobi from zero, in shared memory,
-// one CTA per orbital.  When the coarsest level is level 0 this is the whole
-// preconditioner and the CTA also forms rz and beta.
+// The coarse part of the V-cycle, from each block's first fused level down to
+// its coarsest (40 damped-Jacobi sweeps from zero) and back up, one CTA per
+// orbital with every level in shared memory: two arrays per level with a
+// border of zeros (one point past each row, one row past each plane and a plane
+// on either side, so that every neighbour of a point may be read); r, which
+// becomes the level's correction e in place, and the smoothed residual, later
+// the prolonged iterate.  When the first fused level
+// is level 0 this is the whole preconditioner and the CTA also forms rz and beta.
+//
+// What bounds it: latency (a few thousand points, a barrier between the
+// passes); in float64 one SM's 1.7 FMA per cycle.  A launch per pass spent
+// 5 to 9 us on each level's four kernels whatever the level's size: at 64^3 x 10
+// (levels of 16^3, 8^3 and 4^3 points) 54 us per V-cycle, here 20; at
+// 40^3 x 5 in float64 (10^3 and 5^3) 55, here 37 us.
+constexpr int kMgThreads = 1024;
+
 template <class T>
-__global__ void k_mg_coarsest(const BlkDesc* __restrict__ blk, MgPtrs<T> mp, const int* __restrict__ orb_blk,
-                              int norb, const int* __restrict__ active, T omega, int nsweep, CgState st) {
-    extern __shared__ unsigned char smem_raw[];
-    T* sh = reinterpret_cast<T*>(smem_raw);
+struct MgSm {   // one level in shared memory
+    int nx, ny, nz, px, pxy, G, corr;
+    T h2;
+    const T* w;       // [8] 1 / dd by the dimensions in which the point is last
+    T *r, *s;         // first interior point of the bordered arrays
+};
+
+// inverse diagonal weight at (x, y, z)
+template <class T>
+__device__ __forceinline__ T mg_w(const MgSm<T>& M, int x, int y, int z) {
+    return M.w[(x == M.nx - 1 ? 1 : 0) | (y == M.ny - 1 ? 2 : 0) | (z == M.nz - 1 ? 4 : 0)];
+}
+template <class T>
+__device__ __forceinline__ T mg_nbr(const T* u, const MgSm<T>& M) {
+    return ((u[-1] + u[1]) + (u[-M.px] + u[M.px])) + (u[-M.pxy] + u[M.pxy]);
+}
+template <class T, class Body>
+__device__ __forceinline__ void mg_points(const MgSm<T>& M, Body body) {
+    const int pl = M.nx * M.ny;
+    for (int k = threadIdx.x; k < M.G; k += kMgThreads) {
+        const int z = k / pl, rem = k - z * pl, y = rem / M.nx, x = rem - y * M.nx;
+        body(k, x, y, z, z * M.pxy + y * M.px + x);
+    }
+}
+
+template <class T>
+__global__ void __launch_bounds__(kMgThreads) k_mg_coarse(const BlkDesc* __restrict__ blk, MgPtrs<T> mp,
+                                                          const int* __restrict__ orb_blk, const int* __restrict__ active,
+                                                          T omega, int nsweep, CgState st) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* const sh = reinterpret_cast<T*>(smem_raw);
     __shared__ double scratch[32];
-    const int o = blockIdx.x;
-    if (o >= norb || !active[o]) return;
+    __shared__ MgSm<T> lv[kMaxLevels];
+    __shared__ T s_w[kMaxLevels][8];
+    __shared__ int s_total;
+    const int o = blockIdx.x, tid = threadIdx.x;
+    if (!active[o]) return;
     const int b = orb_blk[o];
-    const int lev = mp.coarsest_level[b];
-    const LvlDesc& D = mp.lvl[lev][b];
+    const int f = mp.fused_level[b], lc = mp.coarsest_level[b];
     const int i = o - blk[b].orb0;
-    const int G = (int)D.G;
-    const long long base = D.off + (long long)i * D.G;
-    const T* r = mp.r[lev] + base;
-    T* e = mp.e[lev] + base;
-    T* rs = sh;
-    T* ea = sh + G;
-    T* eb = sh + 2 * G;
-    const T h2 = T(D.h * D.h);
-    const int pl = D.nx * D.ny;
-    for (int k = threadIdx.x; k < G; k += blockDim.x) {
-        const int z = k / pl, rem = k - z * pl, y = rem / D.nx, x = rem - y * D.nx;
-        rs[k] = r[k];
-        ea[k] = omega * h2 * inv_diag<T>(D, x, y, z) * rs[k];
+    if (tid == 0) {
+        int at = 0;
+        for (int l = f; l <= lc; ++l) {
+            const LvlDesc& D = mp.lvl[l][b];
+            MgSm<T>& M = lv[l];
+            M.nx = D.nx; M.ny = D.ny; M.nz = D.nz;
+            M.px = D.nx + 1;
+            M.pxy = M.px * (D.ny + 1);
+            M.G = (int)D.G;
+            M.corr = D.corr;
+            M.h2 = T(D.h * D.h);
+            M.w = s_w[l];
+            s_w[l][0] = T(1.0 / 6.0);
+            for (int m = 1; m < 8; ++m) s_w[l][m] = T(D.idd[m]);
+            const int pad = M.pxy * (D.nz + 2) + M.px + 1;
+            M.r = sh + at + M.pxy + M.px + 1;
+            M.s = M.r + pad;
+            at += 2 * pad;
+        }
+        s_total = at;
     }
     __syncthreads();
-    for (int sw = 1; sw < nsweep; ++sw) {
-        for (int k = threadIdx.x; k < G; k += blockDim.x) {
-            const int z = k / pl, rem = k - z * pl, y = rem / D.nx, x = rem - y * D.nx;
-            eb[k] = (T(1) - omega) * ea[k] +
-                    omega * inv_diag<T>(D, x, y, z) * (h2 * rs[k] + nbr6(ea, k, x, y, z, D));
+    for (int k = tid; k < s_total; k += kMgThreads) sh[k] = T(0);
+    __syncthreads();
+    const LvlDesc& F = mp.lvl[f][b];
+    const long long base = F.off + (long long)i * F.G;
+    {
+        const T* r = mp.r[f] + base;
+        mg_points(lv[f], [&](int k, int, int, int, int q) { lv[f].r[q] = r[k]; });
+    }
+    __syncthreads();
+    for (int l = f; l < lc; ++l) {
+        const MgSm<T> M = lv[l];
+        const MgSm<T> C = lv[l + 1];
+        // s = r - A2 (omega D^-1 r)
+        mg_points(M, [&](int, int x, int y, int z, int q) {
+            const T* u = M.r + q;
+            T sum;
+            if (M.corr && (x >= M.nx - 2 || y >= M.ny - 2 || z >= M.nz - 2)) {   // a neighbour may lie on a last point
+                sum = u[-1] * mg_w(M, x - 1, y, z) + u[1] * mg_w(M, x + 1, y, z) + u[-M.px] * mg_w(M, x, y - 1, z) +
+                      u[M.px] * mg_w(M, x, y + 1, z) + u[-M.pxy] * mg_w(M, x, y, z - 1) +
+                      u[M.pxy] * mg_w(M, x, y, z + 1);
+            } else {
+                sum = M.w[0] * mg_nbr(u, M);
+            }
+            M.s[q] = (T(1) - omega) * u[0] + omega * sum;
+        });
+        __syncthreads();
+        // full weighting: coarse point I on fine point 2 I + 1
+        mg_points(C, [&](int, int x, int y, int z, int q) {
+            const T* u = M.s + (2 * z + 1) * M.pxy + (2 * y + 1) * M.px + 2 * x + 1;
+            T acc = T(0);
+#pragma unroll
+            for (int c = -1; c <= 1; ++c)
+#pragma unroll
+                for (int a = -1; a <= 1; ++a) {
+                    const T* v = u + c * M.pxy + a * M.px;
+                    acc += (T(c == 0 ? 0.5 : 0.25) * T(a == 0 ? 0.5 : 0.25)) * (T(0.25) * (v[-1] + v[1]) + T(0.5) * v[0]);
+                }
+            C.r[q] = acc;
+        });
+        __syncthreads();
+    }
+    {   // coarsest level: the threads that own points (at most two each) meet at a barrier of their own warps
+        const MgSm<T> M = lv[lc];
+        static_assert(2 * kMgThreads >= kCoarseMax, "points per thread");
+        const int nw = (min(M.G, kMgThreads) + 31) & ~31;
+        if (tid < nw) {
+            int q[2] = {0, 0};
+            T c1[2] = {T(0), T(0)}, c2[2] = {T(0), T(0)};
+            const int pl = M.nx * M.ny;
+            const int np = tid + kMgThreads < M.G ? 2 : (tid < M.G ? 1 : 0);
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+                if (a < np) {
+                    const int k = tid + a * kMgThreads, z = k / pl, rem = k - z * pl, y = rem / M.nx, x = rem - y * M.nx;
+                    q[a] = z * M.pxy + y * M.px + x;
+                    c2[a] = omega * mg_w(M, x, y, z);
+                    c1[a] = c2[a] * M.h2 * M.r[q[a]];
+                }
+            T *ea = M.s, *eb = M.r;   // (r is in the registers now; only its owner reads it)
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+                if (a < np) ea[q[a]] = c1[a];
+            for (int sw = 1; sw < nsweep; ++sw) {
+                asm volatile("bar.sync 1, %0;" ::"r"(nw) : "memory");
+#pragma unroll
+                for (int a = 0; a < 2; ++a)
+                    if (a < np) eb[q[a]] = c2[a] * mg_nbr(ea + q[a], M) + ((T(1) - omega) * ea[q[a]] + c1[a]);
+                T* t = ea; ea = eb; eb = t;
+            }
+            if (ea != M.r) {
+#pragma unroll
+                for (int a = 0; a < 2; ++a)
+                    if (a < np) M.r[q[a]] = ea[q[a]];
+            }
         }
         __syncthreads();
-        T* tmp = ea; ea = eb; eb = tmp;
     }
+    const T* const r0 = mp.r[f] + base;
+    T* const e0 = mp.e[f] + base;
     double rz = 0.0;
-    for (int k = threadIdx.x; k < G; k += blockDim.x) {
-        e[k] = ea[k];
-        rz += (double)rs[k] * (double)ea[k];
+    for (int l = lc - 1; l >= f; --l) {
+        const MgSm<T> M = lv[l];
+        const MgSm<T> C = lv[l + 1];
+        // t = omega D^-1 r + P e_c: per direction an odd point sits on coarse point
+        // (x - 1) / 2, an even one halfway between x / 2 - 1 and x / 2
+        mg_points(M, [&](int, int x, int y, int z, int q) {
+            const int x1 = x >> 1, x0 = x1 - 1 + (x & 1);
+            const int y1 = y >> 1, y0 = y1 - 1 + (y & 1);
+            const int z1 = z >> 1, z0 = z1 - 1 + (z & 1);
+            const T* p00 = C.r + z0 * C.pxy + y0 * C.px;
+            const T* p01 = C.r + z0 * C.pxy + y1 * C.px;
+            const T* p10 = C.r + z1 * C.pxy + y0 * C.px;
+            const T* p11 = C.r + z1 * C.pxy + y1 * C.px;
+            const T u = T(0.125) * (((p00[x0] + p00[x1]) + (p01[x0] + p01[x1])) + ((p10[x0] + p10[x1]) + (p11[x0] + p11[x1])));
+            M.s[q] = omega * M.h2 * (M.corr ? mg_w(M, x, y, z) : M.w[0]) * M.r[q] + u;
+        });
+        __syncthreads();
+        // e = t + omega D^-1 (r - A2 t), in place of r (read by its own point only)
+        mg_points(M, [&](int k, int x, int y, int z, int q) {
+            const T* t = M.s + q;
+            const T w = M.corr ? mg_w(M, x, y, z) : M.w[0];
+            const T e = (T(1) - omega) * t[0] + omega * w * (M.h2 * M.r[q] + mg_nbr(t, M));
+            if (l > f) M.r[q] = e;
+            else e0[k] = e;
+            if (l == 0) rz += (double)M.r[q] * (double)e;
+        });
+        __syncthreads();
     }
-    if (lev == 0) {
+    if (f == lc)   // a single fused level: the sweeps' result
+        mg_points(lv[f], [&](int k, int, int, int, int q) {
+            const T e = lv[f].r[q];
+            if (f == 0) rz += (double)r0[k] * (double)e;
+            e0[k] = e;
+        });
+    if (f == 0) {
         rz = block_sum(rz, scratch);
-        if (threadIdx.x == 0) {
+        if (tid == 0) {
             const double old = st.rz[o];
             st.beta[o] = (old != 0.0) ? rz / old : 0.0;
             st.rz[o] = rz;
@@ -507,13 +656,26 @@ __global__ void k_mg_coarsest(const BlkDesc* __restrict__ blk, MgPtrs<T> mp, con
     }
 }
 
+// Elements of shared memory that k_mg_coarse needs for nlev levels from sides nx, ny, nz on
+long long mg_coarse_elems(int nx, int ny, int nz, int nlev) {
+    long long n = 0;
+    for (int l = 0; l < nlev; ++l) {
+        const long long px = (nx >> l) + 1, pxy = px * ((ny >> l) + 1);
+        n += 2 * (pxy * ((nz >> l) + 2) + px + 1);
+    }
+    return n;
+}
+cudaError_t setup_mg_coarse(const flosic_ctx* c) {
+    return c->opt.precision == FLOSIC_FP64 ? ensure_dyn_smem((const void*)k_mg_coarse<double>, c->mg.coarse_smem)
+                                           : ensure_dyn_smem((const void*)k_mg_coarse<float>, c->mg.coarse_smem);
+}
+
 template <class T>
 void launch_vcycle(const flosic_ctx* c, const MgPtrs<T>& mp, const int* active, cudaStream_t s) {
     const Multigrid& M = c->mg;
     const T omega = T(0.8);
-    const int thr = kChunkThreads;
     const dim3 tb(kTileX, kTileY / 2);
-    for (int l = 0; l + 1 < M.nlev; ++l) {
+    for (int l = 0; l < M.fused_max; ++l) {   // some block's level l is above its fused ones
         if (M.ntiles[l] > 0) {
             k_mg_resid_smooth<T><<<(unsigned)M.ntiles[l], tb, 0, s>>>(c->d_blk, M.d_lvl[l], M.d_tiles[l],
                                                                      c->d_orb_blk, active, mp.r[l], mp.t[l],
@@ -525,10 +687,9 @@ void launch_vcycle(const flosic_ctx* c, const MgPtrs<T>& mp, const int* active, 
                                                                      mp.t[l], mp.r[l + 1]); note_launch(c);
         }
     }
-    const size_t shm = 3 * sizeof(T) * (size_t)M.coarsest_max;
-    k_mg_coarsest<T><<<c->norb, thr, shm, s>>>(c->d_blk, mp, c->d_orb_blk, c->norb, active, omega,
-                                               kCoarseSweeps, c->ws.cg); note_launch(c);
-    for (int l = M.nlev - 2; l >= 0; --l) {
+    k_mg_coarse<T><<<c->norb, kMgThreads, M.coarse_smem, s>>>(c->d_blk, mp, c->d_orb_blk, active, omega, kCoarseSweeps,
+                                                              c->ws.cg); note_launch(c);
+    for (int l = M.fused_max - 1; l >= 0; --l) {
         if (M.ntiles[l] == 0) continue;
         k_mg_prolong<T><<<(unsigned)M.ntiles[l], tb, 0, s>>>(c->d_blk, M.d_lvl[l], M.d_lvl[l + 1],
                                                             M.d_tiles[l], c->d_orb_blk, active, mp.r[l],

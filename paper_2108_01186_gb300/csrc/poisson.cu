@@ -539,6 +539,7 @@ static MgPtrs<T> mg_ptrs(const flosic_ctx* c, T* r, T* z, T* q) {
     mp.e[0] = z;
     mp.t[0] = q;
     mp.coarsest_level = c->mg.d_coarsest_level;
+    mp.fused_level = c->mg.d_fused_level;
     return mp;
 }
 
