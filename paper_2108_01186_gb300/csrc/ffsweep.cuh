@@ -1,6 +1,5 @@
 // 12th-order Laplacian in float-float arithmetic on one 3-D tile (Sec. II.A:
-// high-order centred finite differences), shared by the refinement residual
-// and the mixed-precision Hamiltonian apply.
+// high-order centred finite differences) for the refinement residual.
 //
 // A CTA (32 x 8 threads) owns a 32 x 16 column tile of one orbital and
 // marches along z: per plane the tile plus its 6-point x/y halo is staged in
@@ -32,12 +31,10 @@ static inline cudaError_t upload_ffsweep_weights() {
 // load(g) -> float2 pair of the operand at flat index g (only called for
 // points inside the grid); epi(g, centre, lap) with lap = h^2 Delta_h u at g
 // as a pair, called for every point of the tile inside the grid.
-// kSloppy: the seven weighted terms are accumulated with the two-sum of the
-// high parts and a plain sum of the low parts (error ~ eps^2 times the sum
-// of the terms' magnitudes, ~1e-12 of the result for the smooth potentials
-// of the refinement residual) instead of the renormalised pair addition
-// (error ~ eps^2 of the result, kept for the Hamiltonian apply).
-template <bool kSloppy = false, class Load, class Epi>
+// The seven weighted terms are accumulated with the two-sum of the high parts
+// and a plain sum of the low parts (error ~ eps^2 times the sum of the terms'
+// magnitudes, ~1e-12 of the result for the smooth potentials of the residual).
+template <class Load, class Epi>
 __device__ __forceinline__ void ff_sweep12(const LvlDesc& D, const TilePos& P, Load load, Epi epi,
                                            ff (*plane)[kPX]) {
     const int tx = threadIdx.x, ty = threadIdx.y;
@@ -110,12 +107,8 @@ __device__ __forceinline__ void ff_sweep12(const LvlDesc& D, const TilePos& P, L
                 const ff sm = ff_sum6(plane[ly[k]][lx - m], plane[ly[k]][lx + m], plane[ly[k] - m][lx],
                                       plane[ly[k] + m][lx], qk[kHalf - m], qk[kHalf + m]);
                 const ff tm = ff_mul(w[m], sm);
-                if constexpr (kSloppy) {
-                    const ff s2 = ff_two_sum(acc.h, tm.h);
-                    acc = ff_quick(s2.h, s2.l + (acc.l + tm.l));
-                } else {
-                    acc = ff_add(acc, tm);
-                }
+                const ff s2 = ff_two_sum(acc.h, tm.h);
+                acc = ff_quick(s2.h, s2.l + (acc.l + tm.l));
             }
             if (in[k]) epi(P.base + z * sz + cc[k], qk[kHalf], acc);
         }

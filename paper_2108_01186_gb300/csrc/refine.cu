@@ -20,12 +20,11 @@
 #include <cudaTypedefs.h>
 
 #include "ffsweep.cuh"
+#include "ixsweep.cuh"
 #include "tcgen05.cuh"
 
 namespace flosic {
 
-
-bool ix_weights_match();
 
 // the float-float weights, after checking the update's integer weights
 // against the float64 ones (a mismatch fails the context's creation)
@@ -149,7 +148,7 @@ __global__ void __launch_bounds__(256) k_residual12_ff(const BlkDesc* __restrict
     const BlkDesc& B = blk[P.b];
     const bool padded = B.Gp != B.G;
     float rrf = 0.f;
-    ff_sweep12<true>(
+    ff_sweep12(
         D, P, [&](long long g) { return x[g]; },
         [&](long long g, ff, ff acc) {
             // acc = h^2 Delta_h x, so r = b - A x = b + acc / h^2
@@ -177,46 +176,14 @@ __global__ void __launch_bounds__(256) k_residual12_ff(const BlkDesc* __restrict
 }
 
 // ---------------------------------------------------------------------------
-// Exact stencil sums for the refinement update.  The 12th-order weights of
-// the second derivative (Sec. II.A: centred differences, w_m =
-// 2 (-1)^(m+1) (6!)^2 / (m^2 (6-m)! (6+m)!), w_0 = -2 sum w_m) are rationals
-// whose common denominator is 831600, so W_m = 831600 w_m are integers and
-// h^2 Delta_h u = (1 / 831600) sum_m W_m (sum of the six neighbours at
-// distance m).  A float32 field d whose magnitude is below 2^e splits
-// exactly into y = d 2^(28-e) = hi + lo with hi = rint(y) an integer
-// (|hi| <= 2^28) and |lo| <= 1/2: the hi parts are summed and weighted in
-// integers (six of them stay below 2^31, the weighted sum below 2^53), so
-// that part is exact, and the lo parts in float32, an error of a few units
+// Exact stencil sums for the refinement update (weights W_m: ixsweep.cuh).
+// A float32 field d whose magnitude is below 2^e splits exactly into
+// y = d 2^(28-e) = hi + lo with hi = rint(y) an integer (|hi| <= 2^28) and
+// |lo| <= 1/2: the hi parts are summed and weighted in integers, so that
+// part is exact, and the lo parts in float32, an error of a few units
 // of 2^(e-28) / 831600 in h^2 Delta_h d per point -- about 1e-14 of
 // max |d| / h^2, below the float-float sweep's error on smooth fields.
 // ---------------------------------------------------------------------------
-constexpr long long kW12Den = 831600;
-
-__host__ __device__ constexpr long long w12_fact(int n) { return n <= 1 ? 1 : n * w12_fact(n - 1); }
-__host__ __device__ constexpr long long w12_num(int m) {   // 2 (6!)^2 831600, signed
-    return (m % 2 == 1 ? 2 : -2) * w12_fact(6) * w12_fact(6) * kW12Den;
-}
-__host__ __device__ constexpr long long w12_den(int m) { return (long long)m * m * w12_fact(6 - m) * w12_fact(6 + m); }
-// W_m for m >= 1; W_0 of the three-dimensional centre is 3 (-2 sum_m W_m)
-__host__ __device__ constexpr long long w12_int(int m) { return w12_num(m) / w12_den(m); }
-__host__ __device__ constexpr long long w12_centre3() {
-    return -6 * (w12_int(1) + w12_int(2) + w12_int(3) + w12_int(4) + w12_int(5) + w12_int(6));
-}
-static_assert(w12_num(1) % w12_den(1) == 0 && w12_num(2) % w12_den(2) == 0 && w12_num(3) % w12_den(3) == 0 &&
-                  w12_num(4) % w12_den(4) == 0 && w12_num(5) % w12_den(5) == 0 && w12_num(6) % w12_den(6) == 0,
-              "831600 is a common denominator of the 12th-order weights");
-static_assert(w12_centre3() > -(1LL << 24) && w12_int(1) < (1LL << 24), "weights exact in float32");
-
-// Host check of the integer weights against the float64 ones the other
-// stencils use (|W_m / 831600 - w_m| at rounding level).
-bool ix_weights_match() {
-    double w[kHalf + 1];
-    stencil_weights(w);
-    for (int m = 1; m <= kHalf; ++m)
-        if (std::fabs((double)w12_int(m) / (double)kW12Den - w[m]) > 1e-15 * std::fabs(w[m])) return false;
-    return std::fabs((double)w12_centre3() / (double)kW12Den - 3.0 * w[0]) <= 1e-15 * std::fabs(3.0 * w[0]);
-}
-
 struct __align__(8) IxPt {
     int h;     // rint(y)
     float l;   // y - rint(y), or y itself when it is not finite
@@ -253,17 +220,6 @@ __device__ __forceinline__ IxPt ix_split_w(float d, float s) {
     const float y = d * s;
     const float r = rintf(y);
     return {__float2int_rn(r), y - r};
-}
-
-// ix_to_ff for |I| < 2^53 from I + 2^53 (non-negative): the pieces of 23, 23
-// and 8 bits each exact as floats, the bias removed from the top piece.
-__device__ __forceinline__ ff ix_to_ff_b(long long I, float Lo) {
-    const unsigned long long M = (unsigned long long)I + (1ull << 53);
-    const float f0 = __uint_as_float(0x4B000000u | ((unsigned)M & 0x7fffffu)) - 8388608.f;
-    const float f1 = (__uint_as_float(0x4B000000u | ((unsigned)(M >> 23) & 0x7fffffu)) - 8388608.f) * 8388608.f;
-    const float f2 = (__uint_as_float(0x4B000000u | (unsigned)(M >> 46)) - 8388736.f) * 70368744177664.f;
-    const ff v = ff_two_sum(f2, f1);
-    return ff_two_sum(v.h, (v.l + f0) + Lo);
 }
 
 // Per orbital, max |d| over its grid (float bits in st.dmax, atomicMax on
