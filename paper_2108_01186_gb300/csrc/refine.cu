@@ -26,13 +26,6 @@
 namespace flosic {
 
 
-// the float-float weights, after checking the update's integer weights
-// against the float64 ones (a mismatch fails the context's creation)
-cudaError_t upload_ff_weights() {
-    if (!ix_weights_match()) return cudaErrorInvalidValue;
-    return upload_ffsweep_weights();
-}
-
 // Last CTA of an orbital, once r.r is known: the outer stop test, else the
 // start of the next float32 solve (its target, active flag and counters).
 __device__ __forceinline__ void start_round(CgState& st, int o, double rr, double tol2, double inner_tol2,
@@ -189,33 +182,9 @@ struct __align__(8) IxPt {
     float l;   // y - rint(y), or y itself when it is not finite
 };
 
-// y = d 2^es (exact) split into hi + lo; a non-finite y keeps hi = 0 and
-// carries inf / NaN in lo, so it reaches the residual.
-__device__ __forceinline__ IxPt ix_split(float d, float s) {
-    const float y = d * s;
-    const float r = rintf(y);
-    const bool fin = fabsf(y) < 536870912.f;   // 2^29
-    return {fin ? __float2int_rn(r) : 0, fin ? y - r : y};
-}
-
-// I + Lo as a float-float pair (|I| < 2^53): |I| in three pieces of at most 23
-// bits, each turned into a float exactly by the 2^23 bias (integer and float
-// additions only -- no 64-bit conversion, which would run on the float64
-// pipe), summed with a two-sum; Lo is added to the low part (one rounding).
-__device__ __forceinline__ ff ix_to_ff(long long I, float Lo) {
-    const unsigned long long M = I < 0 ? 0ull - (unsigned long long)I : (unsigned long long)I;
-    const float f0 = __uint_as_float(0x4B000000u | ((unsigned)M & 0x7fffffu)) - 8388608.f;
-    const float f1 = (__uint_as_float(0x4B000000u | ((unsigned)(M >> 23) & 0x7fffffu)) - 8388608.f) * 8388608.f;
-    const float f2 = (__uint_as_float(0x4B000000u | (unsigned)(M >> 46)) - 8388608.f) * 70368744177664.f;
-    ff v = ff_two_sum(f2, f1);
-    const float sg = I < 0 ? -1.f : 1.f;
-    v = ff_two_sum(sg * v.h, sg * (v.l + f0) + Lo);
-    return v;
-}
-
-// ix_split without the finiteness test, for sums taken in unsigned (wrapping)
-// integers: a non-finite y still carries inf / NaN in lo, and its saturated
-// integer part only wraps the integer sum, which lo then overrides.
+// y = d 2^es (exact) split into hi + lo, for sums taken in unsigned (wrapping)
+// integers: a non-finite y carries inf / NaN in lo, so it reaches the
+// residual, and its saturated integer part only wraps the integer sum.
 __device__ __forceinline__ IxPt ix_split_w(float d, float s) {
     const float y = d * s;
     const float r = rintf(y);
@@ -250,176 +219,82 @@ __global__ void __launch_bounds__(256) k_dmax(const BlkDesc* __restrict__ blk, c
     if ((linear_tid() & 31) == 0 && m > 0.f) atomicMax(st.dmax + P.o, __float_as_uint(m));
 }
 
+// Scales of the update of an orbital with max |d| (float bits): |d| < 2^(E -
+// 126) with E the biased exponent of max |d|, so y = d 2^es with es = 154 - E
+// (kept within the normal range) has |y| < 2^28; is = 2^-es, and cf turns the
+// weighted sums into Delta_h d.
+struct IxScale {
+    float sc, is;
+    ff cf;
+};
+__device__ __forceinline__ IxScale ix_scale(unsigned dmax, double h) {
+    const int E = (int)((dmax >> 23) & 0xffu);
+    const int es = max(-126, min(126, 154 - E));
+    return {__uint_as_float((unsigned)(es + 127) << 23), __uint_as_float((unsigned)(127 - es) << 23),
+            to_ff(d2ff(ldexp(1.0 / ((double)kW12Den * h * h), -es)))};
+}
+
+// The weighted sums (integer and float parts) of two neighbouring points:
+// pc the first one in the split plane of kPitch columns, q0 and q1 their
+// z-windows with plane z - 6 in slot u.
+template <int kPitch>
+__device__ __forceinline__ void ix_sums2(const IxPt* pc, const IxPt (&q0)[kQ], const IxPt (&q1)[kQ], int u,
+                                         long long& I0, long long& I1, float& L0, float& L1) {
+    constexpr int kWc = (int)w12_centre3();
+    constexpr int kW[kHalf + 1] = {kWc,           (int)w12_int(1), (int)w12_int(2), (int)w12_int(3),
+                                   (int)w12_int(4), (int)w12_int(5), (int)w12_int(6)};
+    IxPt xw[2 * kHalf + 2];   // columns -6 .. 7 of the row, as 7 pairs
+#pragma unroll
+    for (int k2 = 0; k2 < kHalf + 1; ++k2) {
+        const int4 v = *reinterpret_cast<const int4*>(pc - kHalf + 2 * k2);
+        xw[2 * k2] = {v.x, __int_as_float(v.y)};
+        xw[2 * k2 + 1] = {v.z, __int_as_float(v.w)};
+    }
+    const IxPt c0 = q0[u + kHalf], c1 = q1[u + kHalf];
+    I0 = (long long)kW[0] * c0.h;
+    I1 = (long long)kW[0] * c1.h;
+    L0 = (float)kW[0] * c0.l;
+    L1 = (float)kW[0] * c1.l;
+#pragma unroll
+    for (int m = 1; m <= kHalf; ++m) {
+        const int4 uu = *reinterpret_cast<const int4*>(pc - m * kPitch);   // rows -+ m
+        const int4 ww = *reinterpret_cast<const int4*>(pc + m * kPitch);
+        const IxPt a0 = q0[u + kHalf - m], b0 = q0[u + kHalf + m];
+        const IxPt a1 = q1[u + kHalf - m], b1 = q1[u + kHalf + m];
+        const unsigned h0 = (((unsigned)xw[kHalf - m].h + (unsigned)xw[kHalf + m].h) + ((unsigned)uu.x + (unsigned)ww.x)) +
+                            ((unsigned)a0.h + (unsigned)b0.h);
+        const unsigned h1 = (((unsigned)xw[kHalf + 1 - m].h + (unsigned)xw[kHalf + 1 + m].h) +
+                             ((unsigned)uu.z + (unsigned)ww.z)) + ((unsigned)a1.h + (unsigned)b1.h);
+        const float l0 = ((xw[kHalf - m].l + xw[kHalf + m].l) + (__int_as_float(uu.y) + __int_as_float(ww.y))) +
+                         (a0.l + b0.l);
+        const float l1 = ((xw[kHalf + 1 - m].l + xw[kHalf + 1 + m].l) + (__int_as_float(uu.w) + __int_as_float(ww.w))) +
+                         (a1.l + b1.l);
+        I0 += (long long)kW[m] * (int)h0;
+        I1 += (long long)kW[m] * (int)h1;
+        L0 = fmaf((float)kW[m], l0, L0);
+        L1 = fmaf((float)kW[m], l1, L1);
+    }
+}
+
+// r + Delta_h d and x + d of a point (pairs) from its weighted sums
+__device__ __forceinline__ void ix_update(long long I, float Lo, ff cf, float is, IxPt c, float2 r, float2 x, ff& rn,
+                                          ff& xn) {
+    rn = ff_add(to_ff(r), ff_mul(ix_to_ff_b(I, Lo), cf));
+    const ff xs = ff_two_sum(x.x, (__int2float_rn(c.h) + c.l) * is);   // d at the point (exact)
+    xn = ff_quick(xs.h, xs.l + x.y);
+}
+
 // One refinement round's update from the float32 correction d of the inner
 // solve: r -= A d (r in pairs, in place: r_{k+1} = b - A x_{k+1} =
 // r_k - A d_k), x += d (pairs), r32 = float(r), and the next round's start.
 // A d comes from the exact integer sums above, on the tiles of the other
-// 12th-order sweeps (a CTA of 32 x 8 threads owns a 32 x 16 column tile and
-// marches along z: the plane with its 6-point x/y halo staged in shared
-// memory as split values, the 13 z-values of each of its two columns in
-// registers).  d is left as it is (neighbouring tiles read it as halo): this
-// serves inner solvers that overwrite d (the Kronecker-product solve), not
-// those that start from d = 0.
-// kXZ: the first update after a cold start that stored no x (x = 0, not read)
-template <bool kXZ>
-__global__ void __launch_bounds__(256, 2) k_update12_ix(const BlkDesc* __restrict__ blk, const LvlDesc* __restrict__ L,
-                                                     const int4* __restrict__ tiles, const int* __restrict__ orb_blk,
-                                                     float2* __restrict__ r, float2* __restrict__ x,
-                                                     float* __restrict__ r32, const float* __restrict__ d32,
-                                                     double tol2, double inner_tol2, int max_iter, CgState st) {
-    __shared__ IxPt plane[kPY][kPX];
-    __shared__ double scratch[32];
-    const TilePos P = tile_pos(blk, L, tiles, orb_blk, blockIdx.x);
-    if (!st.oactive[P.o] || L[P.b].utma) return;
-    const LvlDesc& D = L[P.b];
-    // |d| < 2^(E - 126) with E the biased exponent of max |d|: scale by
-    // 2^es, es = 154 - E (so |y| < 2^28), kept within the normal range
-    const int E = (int)((st.dmax[P.o] >> 23) & 0xffu);
-    const int es = max(-126, min(126, 154 - E));
-    const float s = __uint_as_float((unsigned)(es + 127) << 23);    // 2^es
-    const float is = __uint_as_float((unsigned)(127 - es) << 23);   // 2^-es
-    const ff cf = to_ff(d2ff(ldexp(1.0 / ((double)kW12Den * D.h * D.h), -es)));   // units -> Delta_h d
-    constexpr int kWc = (int)w12_centre3();
-    constexpr int kW1 = (int)w12_int(1), kW2 = (int)w12_int(2), kW3 = (int)w12_int(3);
-    constexpr int kW4 = (int)w12_int(4), kW5 = (int)w12_int(5), kW6 = (int)w12_int(6);
-    const int kW[kHalf + 1] = {kWc, kW1, kW2, kW3, kW4, kW5, kW6};
-
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int tid = ty * kTileX + tx;
-    const int nthr = kTileX * (kTileY / 2);
-    const long long sy = D.nx, sz = (long long)D.nx * D.ny;
-    const int gx = P.x0 + tx;
-    const int gy0 = P.y0 + ty, gy1 = P.y0 + ty + kTileY / 2;
-    const bool in0 = gx < D.nx && gy0 < D.ny, in1 = gx < D.nx && gy1 < D.ny;
-    const long long c0 = gy0 * sy + gx, c1 = gy1 * sy + gx;
-    // d and r32 hold the block with padded sides: plane and row strides, the orbital's offset
-    const BlkDesc& B = blk[P.b];
-    const int dpx = B.p[0];
-    const long long dsz = (long long)dpx * B.p[1], db = B.poff + (long long)(P.o - B.orb0) * B.Gp;
-    const long long e0 = (long long)gy0 * dpx + gx, e1 = (long long)gy1 * dpx + gx;
-    int soff[kSlots];   // in-plane offsets of this thread's staged points (-1: outside)
-#pragma unroll
-    for (int j = 0; j < kSlots; ++j) {
-        const int e = tid + j * nthr;
-        soff[j] = -1;
-        if (e < kPX * kPY) {
-            const int yy = e / kPX, xx = e - yy * kPX;
-            int px = P.x0 - kHalf + xx, py = P.y0 - kHalf + yy;
-            if (D.per & 1) px = wrap_coord(px, D.nx);
-            if (D.per & 2) py = wrap_coord(py, D.ny);
-            if (px >= 0 && px < D.nx && py >= 0 && py < D.ny) soff[j] = py * dpx + px;
-        }
-    }
-    IxPt q0[2 * kHalf + 1], q1[2 * kHalf + 1];
-    const bool perz = (D.per & 4) != 0;
-#pragma unroll
-    for (int j = 0; j < 2 * kHalf; ++j) {
-        int zz = P.z0 - kHalf + j;
-        if (perz) zz = wrap_coord(zz, D.nz);
-        const bool okz = zz >= 0 && zz < D.nz;
-        q0[j] = ix_split((in0 && okz) ? d32[db + zz * dsz + e0] : 0.f, s);
-        q1[j] = ix_split((in1 && okz) ? d32[db + zz * dsz + e1] : 0.f, s);
-    }
-    float pre[kSlots];
-#pragma unroll
-    for (int j = 0; j < kSlots; ++j) pre[j] = (soff[j] >= 0) ? d32[db + P.z0 * dsz + soff[j]] : 0.f;
-    // r and x of this thread's two points, one plane ahead of their use
-    constexpr bool xz = kXZ;
-    const float2 f0 = make_float2(0.f, 0.f);
-    float4 rx0 = make_float4(0.f, 0.f, 0.f, 0.f), rx1 = rx0;   // (r.h, r.l, x.h, x.l)
-    if (in0) {
-        const float2 rv = r[P.base + P.z0 * sz + c0], xv = xz ? f0 : x[P.base + P.z0 * sz + c0];
-        rx0 = make_float4(rv.x, rv.y, xv.x, xv.y);
-    }
-    if (in1) {
-        const float2 rv = r[P.base + P.z0 * sz + c1], xv = xz ? f0 : x[P.base + P.z0 * sz + c1];
-        rx1 = make_float4(rv.x, rv.y, xv.x, xv.y);
-    }
-    IxPt* flat = &plane[0][0];
-    float rrf = 0.f;
-    for (int z = P.z0; z < P.z1; ++z) {
-#pragma unroll
-        for (int j = 0; j < kSlots; ++j) {
-            const int e = tid + j * nthr;
-            if (e < kPX * kPY) flat[e] = ix_split(pre[j], s);
-        }
-        {
-            int zz = z + kHalf;
-            if (perz) zz = wrap_coord(zz, D.nz);
-            q0[2 * kHalf] = ix_split((in0 && zz < D.nz) ? d32[db + zz * dsz + e0] : 0.f, s);
-            q1[2 * kHalf] = ix_split((in1 && zz < D.nz) ? d32[db + zz * dsz + e1] : 0.f, s);
-        }
-        __syncthreads();
-        float4 nx0 = rx0, nx1 = rx1;
-        if (z + 1 < P.z1) {
-            const long long pz = P.base + (z + 1) * sz;
-#pragma unroll
-            for (int j = 0; j < kSlots; ++j) pre[j] = (soff[j] >= 0) ? d32[db + (z + 1) * dsz + soff[j]] : 0.f;
-            if (in0) {
-                const float2 rv = r[pz + c0], xv = xz ? f0 : x[pz + c0];
-                nx0 = make_float4(rv.x, rv.y, xv.x, xv.y);
-            }
-            if (in1) {
-                const float2 rv = r[pz + c1], xv = xz ? f0 : x[pz + c1];
-                nx1 = make_float4(rv.x, rv.y, xv.x, xv.y);
-            }
-        }
-        const int lx = tx + kHalf;
-        const int ly[2] = {ty + kHalf, ty + kTileY / 2 + kHalf};
-        const bool in[2] = {in0, in1};
-        const long long cc[2] = {c0, c1};
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const IxPt* qk = (k == 0) ? q0 : q1;
-            long long I = (long long)kW[0] * qk[kHalf].h;
-            float Lo = (float)kW[0] * qk[kHalf].l;
-#pragma unroll
-            for (int m = 1; m <= kHalf; ++m) {
-                const IxPt a = plane[ly[k]][lx - m], b = plane[ly[k]][lx + m];
-                const IxPt c = plane[ly[k] - m][lx], d = plane[ly[k] + m][lx];
-                const IxPt e = qk[kHalf - m], f = qk[kHalf + m];
-                const int hs = ((a.h + b.h) + (c.h + d.h)) + (e.h + f.h);
-                const float ls = ((a.l + b.l) + (c.l + d.l)) + (e.l + f.l);
-                I += (long long)kW[m] * hs;
-                Lo = fmaf((float)kW[m], ls, Lo);
-            }
-            if (in[k]) {
-                const long long g = P.base + z * sz + cc[k];
-                // I + Lo in float-float (I's two leading float parts), times 2^-es / (831600 h^2)
-                const ff ad = ff_mul(ix_to_ff(I, Lo), cf);   // Delta_h d, so r - A d = r + ad
-                const float4 rx = (k == 0) ? rx0 : rx1;
-                const ff rn = ff_add(ff{rx.x, rx.y}, ad);
-                const float dc = (__int2float_rn(qk[kHalf].h) + qk[kHalf].l) * is;   // d at the point (exact)
-                const ff xs = ff_two_sum(rx.z, dc);
-                const ff xn = ff_quick(xs.h, xs.l + rx.w);
-                r[g] = make_float2(rn.h, rn.l);
-                x[g] = make_float2(xn.h, xn.l);
-                r32[db + z * dsz + (k == 0 ? e0 : e1)] = rn.h;
-                rrf += rn.h * rn.h;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < 2 * kHalf; ++j) {
-            q0[j] = q0[j + 1];
-            q1[j] = q1[j + 1];
-        }
-        rx0 = nx0;
-        rx1 = nx1;
-    }
-    if (tile_arrive(rrf, st.part, blockIdx.x, st.count + P.o, D.ntile, scratch)) {
-        const double sum = tile_gather(st.part, P.first, D.ntile, scratch);
-        if (linear_tid() == 0) {
-            st.count[P.o] = 0;
-            st.dmax[P.o] = 0u;   // every CTA of the orbital has read it (and xz)
-            st.xz[P.o] = 0;      // x is stored now
-            start_round(st, P.o, sum, tol2, inner_tol2, max_iter);
-        }
-    }
-}
-
-// The same update with its operands staged by the copy engine (blocks
-// whose rows and offset are 16-byte aligned and that have no periodic
+// 12th-order sweeps (a CTA owns a 32 x 16 column tile and marches along z).
+// d is left as it is (neighbouring tiles read it as halo): this serves inner
+// solvers that overwrite d (the Kronecker-product solve), not those that
+// start from d = 0.  kXZ: the first update after a cold start that stored no
+// x (x = 0, not read).
+//
+// This form has its operands staged by the copy engine (blocks whose rows and offset are 16-byte aligned and that have no periodic
 // direction: the zero fill of the copies is the zero ghost value).  A ring
 // of kURing stages runs ahead of the z-march, each holding the plane z of d
 // with its halo (48 x 28: x0 - 8 keeps the copy 16-byte aligned), d at
@@ -462,15 +337,8 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     const int nzt = P.z1 - P.z0;
     constexpr bool xz = kXZ;   // x is zero and not stored yet: its tiles are not copied
-    const int E = (int)((st.dmax[P.o] >> 23) & 0xffu);
-    const int es = max(-126, min(126, 154 - E));
-    const float sc = __uint_as_float((unsigned)(es + 127) << 23);   // 2^es
-    const float is = __uint_as_float((unsigned)(127 - es) << 23);   // 2^-es
-    const ff cf = to_ff(d2ff(ldexp(1.0 / ((double)kW12Den * D.h * D.h), -es)));
-    constexpr int kWc = (int)w12_centre3();
-    constexpr int kW1 = (int)w12_int(1), kW2 = (int)w12_int(2), kW3 = (int)w12_int(3);
-    constexpr int kW4 = (int)w12_int(4), kW5 = (int)w12_int(5), kW6 = (int)w12_int(6);
-    const int kW[kHalf + 1] = {kWc, kW1, kW2, kW3, kW4, kW5, kW6};
+    __shared__ IxScale s_scale;   // one thread's float64 division
+    if (tid == 0) s_scale = ix_scale(st.dmax[P.o], D.h);
     auto issue = [&](int k) {
         uint64_t* b = bar + (k % kURing);
         float* sg = ring + (size_t)(k % kURing) * kUStage;
@@ -487,6 +355,8 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
         for (int k = 0; k < kURing && k < nzt; ++k) issue(k);
     }
     __syncthreads();
+    const float sc = s_scale.sc, is = s_scale.is;
+    const ff cf = s_scale.cf;
     const int tx = threadIdx.x, ty = threadIdx.y;   // 16 x 16
     const int gx = P.x0 + 2 * tx, gy = P.y0 + ty;
     const bool in = gx < D.nx && gy < D.ny;           // nx is even: gx + 1 < nx as well
@@ -496,10 +366,7 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
     const BlkDesc& B = blk[P.b];
     const long long dsz = (long long)B.p[0] * B.p[1];
     const long long dcol = B.poff + (long long)oi * B.Gp + (long long)gy * B.p[0] + gx;
-    // z-windows of the two points as rings of 13 registers: plane z - 6 + j of
-    // step k sits in slot (k + j) mod 13, so nothing moves between planes (the
-    // z-loop is unrolled by 13 to make every slot index a constant)
-    constexpr int kQ = 2 * kHalf + 1;
+    // z-windows of the two points: plane z - 6 + j of step k0 + u in slot u + j
     IxPt q0[kQ], q1[kQ];
 #pragma unroll
     for (int j = 0; j < 2 * kHalf; ++j) {
@@ -511,9 +378,9 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
     }
     float rrf = 0.f;
     const int ly = ty + kHalf, cx = 2 * tx + 8;       // the points' row and first column in the staged plane
-    for (int k0 = 0; k0 < nzt; k0 += kQ) {
+    for (int k0 = 0; k0 < nzt; k0 += kZU) {
 #pragma unroll
-        for (int u = 0; u < kQ; ++u) {
+        for (int u = 0; u < kZU; ++u) {
             const int k = k0 + u;
             if (k >= nzt) break;
             if (!tc_mbar_wait(bar + (k % kURing), (uint32_t)((k / kURing) & 1))) atomicOr(status + 3, 8);
@@ -522,8 +389,8 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
             for (int e = tid; e < kUPlane; e += 256) sp[e] = ix_split_w(sg[e], sc);
             {
                 const float2 hv = *reinterpret_cast<const float2*>(sg + kUPlane + ty * kTileX + 2 * tx);
-                q0[(u + 2 * kHalf) % kQ] = ix_split_w(hv.x, sc);
-                q1[(u + 2 * kHalf) % kQ] = ix_split_w(hv.y, sc);
+                q0[u + 2 * kHalf] = ix_split_w(hv.x, sc);
+                q1[u + 2 * kHalf] = ix_split_w(hv.y, sc);
             }
             // the split plane is written, and every thread has finished plane k - 1: its
             // stage takes plane k - 1 + kURing (the other split plane is free for plane k + 1)
@@ -532,59 +399,26 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
                 tc_fence_proxy_async();
                 issue(k - 1 + kURing);
             }
-            // x-window of row ly, columns cx - 6 .. cx + 7, as 7 pairs
-            IxPt xw[2 * kHalf + 2];
-#pragma unroll
-            for (int k2 = 0; k2 < kHalf + 1; ++k2) {
-                const int4 v = *reinterpret_cast<const int4*>(sp + ly * kUX + cx - kHalf + 2 * k2);
-                xw[2 * k2] = {v.x, __int_as_float(v.y)};
-                xw[2 * k2 + 1] = {v.z, __int_as_float(v.w)};
-            }
-            const IxPt c0 = q0[(u + kHalf) % kQ], c1 = q1[(u + kHalf) % kQ];
-            long long I0 = (long long)kW[0] * c0.h, I1 = (long long)kW[0] * c1.h;
-            float L0 = (float)kW[0] * c0.l, L1 = (float)kW[0] * c1.l;
-#pragma unroll
-            for (int m = 1; m <= kHalf; ++m) {
-                const int4 uu = *reinterpret_cast<const int4*>(sp + (ly - m) * kUX + cx);   // rows ly -+ m
-                const int4 ww = *reinterpret_cast<const int4*>(sp + (ly + m) * kUX + cx);
-                const IxPt a0 = q0[(u + kHalf - m) % kQ], b0 = q0[(u + kHalf + m) % kQ];
-                const IxPt a1 = q1[(u + kHalf - m) % kQ], b1 = q1[(u + kHalf + m) % kQ];
-                const unsigned h0 = (((unsigned)xw[kHalf - m].h + (unsigned)xw[kHalf + m].h) +
-                                     ((unsigned)uu.x + (unsigned)ww.x)) + ((unsigned)a0.h + (unsigned)b0.h);
-                const unsigned h1 = (((unsigned)xw[kHalf + 1 - m].h + (unsigned)xw[kHalf + 1 + m].h) +
-                                     ((unsigned)uu.z + (unsigned)ww.z)) + ((unsigned)a1.h + (unsigned)b1.h);
-                const float l0 = ((xw[kHalf - m].l + xw[kHalf + m].l) +
-                                  (__int_as_float(uu.y) + __int_as_float(ww.y))) + (a0.l + b0.l);
-                const float l1 = ((xw[kHalf + 1 - m].l + xw[kHalf + 1 + m].l) +
-                                  (__int_as_float(uu.w) + __int_as_float(ww.w))) + (a1.l + b1.l);
-                I0 += (long long)kW[m] * (int)h0;
-                I1 += (long long)kW[m] * (int)h1;
-                L0 = fmaf((float)kW[m], l0, L0);
-                L1 = fmaf((float)kW[m], l1, L1);
-            }
+            long long I0, I1;
+            float L0, L1;
+            ix_sums2<kUX>(sp + ly * kUX + cx, q0, q1, u, I0, I1, L0, L1);
             if (in) {
                 const float4 rv = *reinterpret_cast<const float4*>(sg + kUPlane + kUCtr + ty * 2 * kTileX + 4 * tx);
                 const float4 xv = xz ? make_float4(0.f, 0.f, 0.f, 0.f)
                                      : *reinterpret_cast<const float4*>(sg + kUPlane + 3 * kUCtr + ty * 2 * kTileX + 4 * tx);
                 const long long g = P.base + (P.z0 + k) * sz + col;
                 ff rn[2], xn[2];
-#pragma unroll
-                for (int a = 0; a < 2; ++a) {
-                    const long long I = a == 0 ? I0 : I1;
-                    const float Lo = a == 0 ? L0 : L1;
-                    const IxPt qc = a == 0 ? c0 : c1;
-                    const ff ad = ff_mul(ix_to_ff_b(I, Lo), cf);
-                    rn[a] = ff_add(a == 0 ? ff{rv.x, rv.y} : ff{rv.z, rv.w}, ad);
-                    const float dc = (__int2float_rn(qc.h) + qc.l) * is;
-                    const ff xs = ff_two_sum(a == 0 ? xv.x : xv.z, dc);
-                    xn[a] = ff_quick(xs.h, xs.l + (a == 0 ? xv.y : xv.w));
-                    rrf += rn[a].h * rn[a].h;
-                }
+                ix_update(I0, L0, cf, is, q0[u + kHalf], make_float2(rv.x, rv.y), make_float2(xv.x, xv.y), rn[0], xn[0]);
+                ix_update(I1, L1, cf, is, q1[u + kHalf], make_float2(rv.z, rv.w), make_float2(xv.z, xv.w), rn[1], xn[1]);
+                rrf += rn[0].h * rn[0].h;
+                rrf += rn[1].h * rn[1].h;
                 *reinterpret_cast<float4*>(r + g) = make_float4(rn[0].h, rn[0].l, rn[1].h, rn[1].l);
                 *reinterpret_cast<float4*>(x + g) = make_float4(xn[0].h, xn[0].l, xn[1].h, xn[1].l);
                 *reinterpret_cast<float2*>(r32 + (P.z0 + k) * dsz + dcol) = make_float2(rn[0].h, rn[1].h);
             }
         }
+        ix_shift(q0);
+        ix_shift(q1);
     }
     if (tile_arrive(rrf, st.part, blockIdx.x, st.count + P.o, D.ntile, scratch)) {
         const double sum = tile_gather(st.part, P.first, D.ntile, scratch);
@@ -597,11 +431,188 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
     }
 }
 
+// The same update for the other blocks (odd rows, rows or offsets off 16
+// bytes, periodic directions).  d's planes arrive by asynchronous copies
+// (IxStage), r and x by 8-byte copies one plane ahead; one barrier per plane.
+// What bounds it: instruction issue, as above.  The plain-load sweep it
+// replaced (two barriers per plane, 24 eight-byte shared loads per point, its
+// z-windows moved every plane) took 1149 us for the two updates of 117^3 x 20,
+// this one about 1000 us.
+constexpr int kCOffRx = kIxPts * 8 * kIxRing;
+constexpr int kCSmem = kCOffRx + 2 * 16 * kUCtr;     // two stages of r and x pairs
+
+template <bool kXZ>
+__global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restrict__ blk, const LvlDesc* __restrict__ L,
+                                                        const int4* __restrict__ tiles, const int* __restrict__ orb_blk,
+                                                        const float* __restrict__ d32, float2* __restrict__ r,
+                                                        float2* __restrict__ x, float* __restrict__ r32, double tol2,
+                                                        double inner_tol2, int max_iter, CgState st) {
+    extern __shared__ __align__(16) unsigned char uc_raw[];
+    IxPt* const ring = reinterpret_cast<IxPt*>(uc_raw);
+    float2* const rx = reinterpret_cast<float2*>(uc_raw + kCOffRx);   // [2][r, x][kUCtr]
+    __shared__ double scratch[32];
+    const TilePos P = tile_pos(blk, L, tiles, orb_blk, blockIdx.x);
+    if (!st.oactive[P.o] || L[P.b].utma) return;
+    const LvlDesc& D = L[P.b];
+    const BlkDesc& B = blk[P.b];
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    const int nx = D.nx, ny = D.ny, nz = D.nz, per = D.per;
+    __shared__ IxScale s_scale;   // one thread's float64 division
+    if (tid == 0) s_scale = ix_scale(st.dmax[P.o], D.h);
+    const long long sy = nx, sz = (long long)nx * ny;
+    // d and r32 hold the block with padded sides
+    const int dpx = B.p[0];
+    const long long dsz = (long long)dpx * B.p[1], db = B.poff + (long long)(P.o - B.orb0) * B.Gp;
+    IxStage sg;
+    sg.init(D, P, dpx, tid);
+    const bool vec = (dpx & 1) == 0 && (db & 1) == 0 && (per & 1) == 0;
+    const int nzt = P.z1 - P.z0;
+    auto copy_d = [&](int k, int slot) {   // plane z0 + k
+        int z = P.z0 + k;
+        if (per & 4) z = wrap_coord(z, nz);
+        const bool okz = z < nz;
+        const float* pl = d32 + db + (okz ? z * dsz : 0);
+#pragma unroll
+        for (int j = 0; j < kIxU; ++j)
+            if (sg.wants(j, k < nzt)) sg.copy(j, ring + slot * kIxPts + 2 * (tid + j * 256), pl, okz, vec, nx);
+    };
+    auto split = [&](int k, int slot, float sc) {
+#pragma unroll
+        for (int j = 0; j < kIxU; ++j)
+            if (sg.wants(j, k < nzt)) {
+                IxPt* const at = ring + slot * kIxPts + 2 * (tid + j * 256);
+                const float2 v = *reinterpret_cast<const float2*>(at);
+                const IxPt a = ix_split_w(v.x, sc), b = ix_split_w(v.y, sc);
+                *reinterpret_cast<int4*>(at) = make_int4(a.h, __float_as_int(a.l), b.h, __float_as_int(b.l));
+            }
+    };
+    // r and x of plane z0 + k: rows of 32 points per warp
+    const int cxp = P.x0 + (tid & 31), cyp = P.y0 + (tid >> 5);
+    auto copy_rx = [&](int k) {
+        float2* const dst = rx + (k & 1) * 2 * kUCtr + tid;
+        const long long g0 = P.base + (P.z0 + k) * sz;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const bool ok = cxp < nx && cyp + 8 * j < ny;
+            const long long g = g0 + (ok ? (cyp + 8 * j) * sy + cxp : 0);
+            cp_async<8>(dst + 256 * j, r + g, ok ? 8 : 0);
+            if (!kXZ) cp_async<8>(dst + kUCtr + 256 * j, x + g, ok ? 8 : 0);
+        }
+    };
+    for (int k = 0; k < kHalf; ++k) copy_d(k, k);
+    copy_rx(0);
+    cp_async_commit();
+    copy_d(kHalf, kHalf);
+    cp_async_commit();
+    copy_d(kHalf + 1, kHalf + 1);
+    cp_async_commit();
+
+    const int tx = threadIdx.x, ty = threadIdx.y;     // 16 x 16; points (x0 + 2 tx + a, y0 + ty)
+    const int gx = P.x0 + 2 * tx, gy = P.y0 + ty;
+    const bool in0 = gx < nx && gy < ny, in1 = gx + 1 < nx && gy < ny;
+    const long long col = gy * sy + gx, dcol = db + (long long)gy * dpx + gx;
+    const int ctr = (ty + kHalf) * kPX + 2 * tx + kHalf;   // the first point in a staged plane
+    __syncthreads();
+    const float sc = s_scale.sc, is = s_scale.is;
+    const ff cf = s_scale.cf;
+    IxPt q0[kQ], q1[kQ];   // z-windows: step k0 + u's in slots u .. u + 12
+#pragma unroll
+    for (int j = 0; j < kHalf; ++j) {   // planes z0 - 6 .. z0 - 1 straight from memory
+        int z = P.z0 - kHalf + j;
+        if (per & 4) z = wrap_coord(z, nz);
+        const float* pl = d32 + z * dsz + dcol;
+        q0[j] = ix_split_w(z >= 0 && z < nz && in0 ? pl[0] : 0.f, sc);
+        q1[j] = ix_split_w(z >= 0 && z < nz && in1 ? pl[1] : 0.f, sc);
+    }
+    asm volatile("cp.async.wait_group 2;" ::: "memory");
+    for (int k = 0; k < kHalf; ++k) split(k, k, sc);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kHalf; ++k) {
+        const int4 hv = *reinterpret_cast<const int4*>(ring + k * kIxPts + ctr);
+        q0[kHalf + k] = {hv.x, __int_as_float(hv.y)};
+        q1[kHalf + k] = {hv.z, __int_as_float(hv.w)};
+    }
+    float rrf = 0.f;
+    int slot = 0;   // of plane z0 + k
+    for (int k0 = 0; k0 < nzt; k0 += kZU) {
+#pragma unroll
+        for (int u = 0; u < kZU; ++u) {
+            const int k = k0 + u;
+            if (k >= nzt) break;
+            // the slot of plane k + 8 held plane k - 2, which every thread has finished; all
+            // but that copy have arrived (the planes up to k + 7, plane k's r and x)
+            if (k + 2 < nzt) copy_d(k + kHalf + 2, ix_slot(slot, kHalf + 2));
+            cp_async_commit();
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            const int hslot = ix_slot(slot, kHalf);
+            split(k + kHalf, hslot, sc);
+            // plane k + 6 is split, and every thread has finished plane k - 1, whose stage of
+            // r and x takes plane k + 1's
+            __syncthreads();
+            if (k + 1 < nzt) copy_rx(k + 1);
+            cp_async_commit();
+            {
+                const int4 hv = *reinterpret_cast<const int4*>(ring + hslot * kIxPts + ctr);
+                q0[u + 2 * kHalf] = {hv.x, __int_as_float(hv.y)};
+                q1[u + 2 * kHalf] = {hv.z, __int_as_float(hv.w)};
+            }
+            const IxPt* const pc = ring + slot * kIxPts + ctr;
+            slot = ix_slot(slot, 1);
+            long long I0, I1;
+            float L0, L1;
+            ix_sums2<kPX>(pc, q0, q1, u, I0, I1, L0, L1);
+            const float2* const st2 = rx + (k & 1) * 2 * kUCtr + ty * kTileX + 2 * tx;
+            const float4 rv = *reinterpret_cast<const float4*>(st2);
+            const float4 xv = kXZ ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(st2 + kUCtr);
+            ff rn[2], xn[2];
+            ix_update(I0, L0, cf, is, q0[u + kHalf], make_float2(rv.x, rv.y), make_float2(xv.x, xv.y), rn[0], xn[0]);
+            ix_update(I1, L1, cf, is, q1[u + kHalf], make_float2(rv.z, rv.w), make_float2(xv.z, xv.w), rn[1], xn[1]);
+            const int z = P.z0 + k;
+            const long long g = P.base + z * sz + col;
+            if (in0) {
+                r[g] = make_float2(rn[0].h, rn[0].l);
+                x[g] = make_float2(xn[0].h, xn[0].l);
+                r32[z * dsz + dcol] = rn[0].h;
+                rrf += rn[0].h * rn[0].h;
+            }
+            if (in1) {
+                r[g + 1] = make_float2(rn[1].h, rn[1].l);
+                x[g + 1] = make_float2(xn[1].h, xn[1].l);
+                r32[z * dsz + dcol + 1] = rn[1].h;
+                rrf += rn[1].h * rn[1].h;
+            }
+        }
+        ix_shift(q0);
+        ix_shift(q1);
+    }
+    if (tile_arrive(rrf, st.part, blockIdx.x, st.count + P.o, D.ntile, scratch)) {
+        const double sum = tile_gather(st.part, P.first, D.ntile, scratch);
+        if (linear_tid() == 0) {
+            st.count[P.o] = 0;
+            st.dmax[P.o] = 0u;   // every CTA of the orbital has read it (and xz)
+            st.xz[P.o] = 0;      // x is stored now
+            start_round(st, P.o, sum, tol2, inner_tol2, max_iter);
+        }
+    }
+}
+
+// The float-float weights, after checking the update's integer weights
+// against the float64 ones (a mismatch fails the context's creation), and the
+// shared memory of the update that needs no tensor maps.
+cudaError_t upload_ff_weights() {
+    if (!ix_weights_match()) return cudaErrorInvalidValue;
+    cudaError_t e = ensure_dyn_smem((const void*)k_update12_cp<false>, kCSmem);
+    if (e == cudaSuccess) e = ensure_dyn_smem((const void*)k_update12_cp<true>, kCSmem);
+    if (e != cudaSuccess) return e;
+    return upload_ffsweep_weights();
+}
+
 // Tensor maps of the update's operands, four per block, each a 4-D view
 // (x, y, z, orbital): d with 48 x 28 boxes and 32 x 16 boxes, and the pair
 // arrays r (b) and x as float32 rows of 2 nx values with 64 x 16 boxes.
 // Blocks with a periodic direction, or whose rows or offset are not
-// 16-byte aligned, keep k_update12_ix (flag utma = 0).  Returns the number
+// 16-byte aligned, take k_update12_cp (flag utma = 0).  Returns the number
 // of blocks on the copy-engine path.
 int setup_update_maps(flosic_ctx* c) {
     void* fn = nullptr;
@@ -750,10 +761,10 @@ void launch_update_ff(flosic_ctx* c, double* r, float2* x, bool x_zero, double t
             reinterpret_cast<float2*>(r), x, c->ws.r32, tol2, inner_tol2, c->opt.max_iter, c->ws.cg, c->ws.status);
         note_launch(c);
     }
-    if (c->n_utma_blocks < c->nblk) {   // the rest: plain loads
-        auto kern = x_zero ? k_update12_ix<true> : k_update12_ix<false>;
-        kern<<<(unsigned)M.ntiles[0], tile_threads(), 0, s>>>(
-            c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, reinterpret_cast<float2*>(r), x, c->ws.r32, c->ws.d32,
+    if (c->n_utma_blocks < c->nblk) {   // the rest: asynchronous copies of single points
+        auto kern = x_zero ? k_update12_cp<true> : k_update12_cp<false>;
+        kern<<<(unsigned)M.ntiles[0], dim3(kTileX / 2, kTileY), kCSmem, s>>>(
+            c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, c->ws.d32, reinterpret_cast<float2*>(r), x, c->ws.r32,
             tol2, inner_tol2, c->opt.max_iter, c->ws.cg);
         note_launch(c);
     }
