@@ -400,9 +400,9 @@ void launch_residual_ff(flosic_ctx* c, const double* b, const float2* x, float* 
                         double inner_tol2, bool store_r, cudaStream_t s);
 void launch_correct_ff(flosic_ctx* c, float2* x, cudaStream_t s);
 // Kronecker inner solver: x += d and r -= A d in one sweep (r in pairs over b)
-void launch_update_ff(flosic_ctx* c, double* r, float2* x, bool x_zero, double tol2, double inner_tol2,
+void launch_update_ff(flosic_ctx* c, double* r, float2* x, double* V, bool x_zero, double tol2, double inner_tol2,
                       cudaStream_t s);
-void launch_join_ff(flosic_ctx* c, const float2* x, double* V, cudaStream_t s);
+void launch_join_ff(flosic_ctx* c, const float2* x, bool kron, bool warm, double* V, cudaStream_t s);
 void stencil_weights(double* w);   // 12th-order weights w_0..w_6
 const void* k_lowdin_symbol();
 int check_cuda(flosic_ctx* c, cudaError_t e, const char* what);

@@ -676,12 +676,12 @@ int run_poisson(flosic_ctx* c, double* b, double* V, bool warm, cudaStream_t s) 
             if (fused) {
                 if (check_cuda(c, cudaMemsetAsync(st.n_active, 0, sizeof(int), s), "memset"))
                     return FLOSIC_ERR_CUDA;
-                launch_update_ff(c, b, x, round == 0 && !warm, tol2, inner_tol2, s);
+                launch_update_ff(c, b, x, V, round == 0 && !warm, tol2, inner_tol2, s);
             } else {
                 launch_correct_ff(c, x, s);
             }
         }
-        launch_join_ff(c, x, V, s);
+        launch_join_ff(c, x, fused, warm, V, s);
     }
     if (c->n_unmasked < c->norb) {
         k_zero_masked<<<nb, T, 0, s>>>(c->d_blk, c->d_chunk_orb, c->d_orb_blk, st.mask, V);

@@ -276,12 +276,14 @@ __device__ __forceinline__ void ix_sums2(const IxPt* pc, const IxPt (&q0)[kQ], c
     }
 }
 
-// r + Delta_h d and x + d of a point (pairs) from its weighted sums
-__device__ __forceinline__ void ix_update(long long I, float Lo, ff cf, float is, IxPt c, float2 r, float2 x, ff& rn,
-                                          ff& xn) {
-    rn = ff_add(to_ff(r), ff_mul(ix_to_ff_b(I, Lo), cf));
-    const ff xs = ff_two_sum(x.x, (__int2float_rn(c.h) + c.l) * is);   // d at the point (exact)
-    xn = ff_quick(xs.h, xs.l + x.y);
+// r + Delta_h d (pairs) of a point from its weighted sums, and d there (exact)
+__device__ __forceinline__ ff ix_update(long long I, float Lo, ff cf, float2 r) {
+    return ff_add(to_ff(r), ff_mul(ix_to_ff_b(I, Lo), cf));
+}
+__device__ __forceinline__ float ix_centre(IxPt c, float is) { return (__int2float_rn(c.h) + c.l) * is; }
+__device__ __forceinline__ ff ix_add(float2 x, float d) {   // x + d
+    const ff s = ff_two_sum(x.x, d);
+    return ff_quick(s.h, s.l + x.y);
 }
 
 // One refinement round's update from the float32 correction d of the inner
@@ -407,9 +409,9 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
                 const float4 xv = xz ? make_float4(0.f, 0.f, 0.f, 0.f)
                                      : *reinterpret_cast<const float4*>(sg + kUPlane + 3 * kUCtr + ty * 2 * kTileX + 4 * tx);
                 const long long g = P.base + (P.z0 + k) * sz + col;
-                ff rn[2], xn[2];
-                ix_update(I0, L0, cf, is, q0[u + kHalf], make_float2(rv.x, rv.y), make_float2(xv.x, xv.y), rn[0], xn[0]);
-                ix_update(I1, L1, cf, is, q1[u + kHalf], make_float2(rv.z, rv.w), make_float2(xv.z, xv.w), rn[1], xn[1]);
+                const ff rn[2] = {ix_update(I0, L0, cf, make_float2(rv.x, rv.y)), ix_update(I1, L1, cf, make_float2(rv.z, rv.w))};
+                const ff xn[2] = {ix_add(make_float2(xv.x, xv.y), ix_centre(q0[u + kHalf], is)),
+                                  ix_add(make_float2(xv.z, xv.w), ix_centre(q1[u + kHalf], is))};
                 rrf += rn[0].h * rn[0].h;
                 rrf += rn[1].h * rn[1].h;
                 *reinterpret_cast<float4*>(r + g) = make_float4(rn[0].h, rn[0].l, rn[1].h, rn[1].l);
@@ -433,23 +435,27 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
 
 // The same update for the other blocks (odd rows, rows or offsets off 16
 // bytes, periodic directions).  d's planes arrive by asynchronous copies
-// (IxStage), r and x by 8-byte copies one plane ahead; one barrier per plane.
+// (IxStage), r and V by 8-byte copies one plane ahead; one barrier per plane.
+// x is the caller's float64 V itself, V += d: a conversion and one float64
+// addition per point, and no pass joins pairs into V at the end (117^3 x 20
+// 2.60 -> 2.44 ms, an uneven batch 6.40 -> 6.06 ms).  k_update12_tma keeps pairs:
+// with V its two launches at 128^3 x 64 grew by more than the 0.35 ms of the join.
 // What bounds it: instruction issue, as above.  The plain-load sweep it
 // replaced (two barriers per plane, 24 eight-byte shared loads per point, its
 // z-windows moved every plane) took 1149 us for the two updates of 117^3 x 20,
 // this one about 1000 us.
 constexpr int kCOffRx = kIxPts * 8 * kIxRing;
-constexpr int kCSmem = kCOffRx + 2 * 16 * kUCtr;     // two stages of r and x pairs
+constexpr int kCSmem = kCOffRx + 2 * 16 * kUCtr;     // two stages of r and V
 
 template <bool kXZ>
 __global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restrict__ blk, const LvlDesc* __restrict__ L,
                                                         const int4* __restrict__ tiles, const int* __restrict__ orb_blk,
                                                         const float* __restrict__ d32, float2* __restrict__ r,
-                                                        float2* __restrict__ x, float* __restrict__ r32, double tol2,
+                                                        double* __restrict__ V, float* __restrict__ r32, double tol2,
                                                         double inner_tol2, int max_iter, CgState st) {
     extern __shared__ __align__(16) unsigned char uc_raw[];
     IxPt* const ring = reinterpret_cast<IxPt*>(uc_raw);
-    float2* const rx = reinterpret_cast<float2*>(uc_raw + kCOffRx);   // [2][r, x][kUCtr]
+    float2* const rx = reinterpret_cast<float2*>(uc_raw + kCOffRx);   // [2][r pairs, V][kUCtr]
     __shared__ double scratch[32];
     const TilePos P = tile_pos(blk, L, tiles, orb_blk, blockIdx.x);
     if (!st.oactive[P.o] || L[P.b].utma) return;
@@ -486,7 +492,7 @@ __global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restric
                 *reinterpret_cast<int4*>(at) = make_int4(a.h, __float_as_int(a.l), b.h, __float_as_int(b.l));
             }
     };
-    // r and x of plane z0 + k: rows of 32 points per warp
+    // r and V of plane z0 + k: rows of 32 points per warp
     const int cxp = P.x0 + (tid & 31), cyp = P.y0 + (tid >> 5);
     auto copy_rx = [&](int k) {
         float2* const dst = rx + (k & 1) * 2 * kUCtr + tid;
@@ -496,7 +502,7 @@ __global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restric
             const bool ok = cxp < nx && cyp + 8 * j < ny;
             const long long g = g0 + (ok ? (cyp + 8 * j) * sy + cxp : 0);
             cp_async<8>(dst + 256 * j, r + g, ok ? 8 : 0);
-            if (!kXZ) cp_async<8>(dst + kUCtr + 256 * j, x + g, ok ? 8 : 0);
+            if (!kXZ) cp_async<8>(dst + kUCtr + 256 * j, V + g, ok ? 8 : 0);
         }
     };
     for (int k = 0; k < kHalf; ++k) copy_d(k, k);
@@ -541,14 +547,14 @@ __global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restric
             const int k = k0 + u;
             if (k >= nzt) break;
             // the slot of plane k + 8 held plane k - 2, which every thread has finished; all
-            // but that copy have arrived (the planes up to k + 7, plane k's r and x)
+            // but that copy have arrived (the planes up to k + 7, plane k's r and V)
             if (k + 2 < nzt) copy_d(k + kHalf + 2, ix_slot(slot, kHalf + 2));
             cp_async_commit();
             asm volatile("cp.async.wait_group 1;" ::: "memory");
             const int hslot = ix_slot(slot, kHalf);
             split(k + kHalf, hslot, sc);
             // plane k + 6 is split, and every thread has finished plane k - 1, whose stage of
-            // r and x takes plane k + 1's
+            // r and V takes plane k + 1's
             __syncthreads();
             if (k + 1 < nzt) copy_rx(k + 1);
             cp_async_commit();
@@ -564,21 +570,24 @@ __global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restric
             ix_sums2<kPX>(pc, q0, q1, u, I0, I1, L0, L1);
             const float2* const st2 = rx + (k & 1) * 2 * kUCtr + ty * kTileX + 2 * tx;
             const float4 rv = *reinterpret_cast<const float4*>(st2);
-            const float4 xv = kXZ ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(st2 + kUCtr);
-            ff rn[2], xn[2];
-            ix_update(I0, L0, cf, is, q0[u + kHalf], make_float2(rv.x, rv.y), make_float2(xv.x, xv.y), rn[0], xn[0]);
-            ix_update(I1, L1, cf, is, q1[u + kHalf], make_float2(rv.z, rv.w), make_float2(xv.z, xv.w), rn[1], xn[1]);
+            const ff rn[2] = {ix_update(I0, L0, cf, make_float2(rv.x, rv.y)), ix_update(I1, L1, cf, make_float2(rv.z, rv.w))};
+            double2 vn = make_double2(f2d(ix_centre(q0[u + kHalf], is)), f2d(ix_centre(q1[u + kHalf], is)));
+            if (!kXZ) {
+                const double2 vo = *reinterpret_cast<const double2*>(st2 + kUCtr);
+                vn.x += vo.x;
+                vn.y += vo.y;
+            }
             const int z = P.z0 + k;
             const long long g = P.base + z * sz + col;
             if (in0) {
                 r[g] = make_float2(rn[0].h, rn[0].l);
-                x[g] = make_float2(xn[0].h, xn[0].l);
+                V[g] = vn.x;
                 r32[z * dsz + dcol] = rn[0].h;
                 rrf += rn[0].h * rn[0].h;
             }
             if (in1) {
                 r[g + 1] = make_float2(rn[1].h, rn[1].l);
-                x[g + 1] = make_float2(xn[1].h, xn[1].l);
+                V[g + 1] = vn.y;
                 r32[z * dsz + dcol + 1] = rn[1].h;
                 rrf += rn[1].h * rn[1].h;
             }
@@ -591,7 +600,7 @@ __global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restric
         if (linear_tid() == 0) {
             st.count[P.o] = 0;
             st.dmax[P.o] = 0u;   // every CTA of the orbital has read it (and xz)
-            st.xz[P.o] = 0;      // x is stored now
+            st.xz[P.o] = 0;      // V is stored now
             start_round(st, P.o, sum, tol2, inner_tol2, max_iter);
         }
     }
@@ -698,13 +707,25 @@ __global__ void __launch_bounds__(256) k_correct_ff(const BlkDesc* __restrict__ 
     });
 }
 
-// V = x (pairs joined into float64), every orbital.
+// V = 0 for the orbitals of k_update12_cp's blocks that it never updated (no solve needed).
+__global__ void __launch_bounds__(256) k_zero_unsolved(const BlkDesc* __restrict__ blk, const LvlDesc* __restrict__ L,
+                                                       const int* __restrict__ orb_blk, const int* __restrict__ xz,
+                                                       double* __restrict__ V) {
+    const int o = blockIdx.x, b = orb_blk[o];
+    if (!xz[o] || L[b].utma) return;
+    const BlkDesc& B = blk[b];
+    double* v = V + B.off + (long long)(o - B.orb0) * B.G;
+    for (long long g = (long long)blockIdx.y * 256 + threadIdx.x; g < B.G; g += 256LL * gridDim.y) v[g] = 0.0;
+}
+
+// V = x (pairs joined into float64), every orbital (utma: of the blocks of k_update12_tma).
 __global__ void __launch_bounds__(256) k_join_ff(const BlkDesc* __restrict__ blk, const LvlDesc* __restrict__ L,
                                                  const int4* __restrict__ tiles, const int* __restrict__ orb_blk,
                                                  const float2* __restrict__ x, const int* __restrict__ xz,
-                                                 double* __restrict__ V) {
+                                                 int utma, double* __restrict__ V) {
     const TilePos P = tile_pos(blk, L, tiles, orb_blk, blockIdx.x);
     const LvlDesc& D = L[P.b];
+    if (utma && !D.utma) return;
     if (xz[P.o]) {   // never updated (no solve needed): V = 0
         tile_elementwise<float>(D, P, [&](long long g, int n) {
             for (int k = 0; k < n; ++k) V[g + k] = 0.0;
@@ -746,7 +767,7 @@ void launch_residual_ff(flosic_ctx* c, const double* b, const float2* x, float* 
 }
 
 // x_zero: the first update after a cold start that stored no x
-void launch_update_ff(flosic_ctx* c, double* r, float2* x, bool x_zero, double tol2, double inner_tol2,
+void launch_update_ff(flosic_ctx* c, double* r, float2* x, double* V, bool x_zero, double tol2, double inner_tol2,
                       cudaStream_t s) {
     const Multigrid& M = c->mg;
     if (c->kron.n_simt > 0) {   // the tensor-core passes record max |d| themselves
@@ -761,10 +782,10 @@ void launch_update_ff(flosic_ctx* c, double* r, float2* x, bool x_zero, double t
             reinterpret_cast<float2*>(r), x, c->ws.r32, tol2, inner_tol2, c->opt.max_iter, c->ws.cg, c->ws.status);
         note_launch(c);
     }
-    if (c->n_utma_blocks < c->nblk) {   // the rest: asynchronous copies of single points
+    if (c->n_utma_blocks < c->nblk) {   // the rest: asynchronous copies, x = V
         auto kern = x_zero ? k_update12_cp<true> : k_update12_cp<false>;
         kern<<<(unsigned)M.ntiles[0], dim3(kTileX / 2, kTileY), kCSmem, s>>>(
-            c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, c->ws.d32, reinterpret_cast<float2*>(r), x, c->ws.r32,
+            c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, c->ws.d32, reinterpret_cast<float2*>(r), V, c->ws.r32,
             tol2, inner_tol2, c->opt.max_iter, c->ws.cg);
         note_launch(c);
     }
@@ -777,11 +798,19 @@ void launch_correct_ff(flosic_ctx* c, float2* x, cudaStream_t s) {
     note_launch(c);
 }
 
-void launch_join_ff(flosic_ctx* c, const float2* x, double* V, cudaStream_t s) {
+// After the rounds: V = x.  The Kronecker rounds (kron) of k_update12_cp's blocks left V
+// complete but for orbitals never updated from a cold start.
+void launch_join_ff(flosic_ctx* c, const float2* x, bool kron, bool warm, double* V, cudaStream_t s) {
     const Multigrid& M = c->mg;
-    k_join_ff<<<(unsigned)M.ntiles[0], tile_threads(), 0, s>>>(c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, x,
-                                                               c->ws.cg.xz, V);
-    note_launch(c);
+    if (!kron || c->n_utma_blocks > 0) {
+        k_join_ff<<<(unsigned)M.ntiles[0], tile_threads(), 0, s>>>(c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, x,
+                                                                   c->ws.cg.xz, kron ? 1 : 0, V);
+        note_launch(c);
+    }
+    if (kron && !warm && c->n_utma_blocks < c->nblk) {
+        k_zero_unsolved<<<dim3(c->norb, 16), 256, 0, s>>>(c->d_blk, M.d_lvl[0], c->d_orb_blk, c->ws.cg.xz, V);
+        note_launch(c);
+    }
 }
 
 }  // namespace flosic
