@@ -272,8 +272,8 @@ int flosic_sic_backward(flosic_ctx* ctx, const double* psi, const double* fods,
  *      potential as written by flosic_sic_energy_potential (scaled by s).
  * Out: Hpsi [sum N*G] float64 (must not overlap psi).
  * Precision follows the context: FP64 in float64; MIXED with the Laplacian
- * and the potential term in float-float pairs (~48 bits), no float64
- * arithmetic per point but the final sum.
+ * in exact integer sums of psi held to 2^-57 of the largest value nearby, the
+ * potential term in float64.
  * Errors: ARG (NULL ctx, psi or Hpsi, or Hpsi == psi), CUDA.  Asynchronous
  * on `stream`. */
 int flosic_hamiltonian_apply(flosic_ctx* ctx, const double* psi, const double* vloc,

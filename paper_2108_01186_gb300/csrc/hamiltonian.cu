@@ -347,11 +347,11 @@ void launch_hamiltonian(const flosic_ctx* c, const double* psi, const double* vl
     const Multigrid& M = c->mg;
     const dim3 tb(kTileX, kTileY / 2);
     if (c->opt.precision == FLOSIC_MIXED) {
-        int* texp = reinterpret_cast<int*>(c->ws.cg.part);   // one per tile (scratch of the solves)
-        k_tile_exp<<<(unsigned)M.ntiles[0], tb, 0, s>>>(c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, psi, texp);
+        k_tile_exp<<<(unsigned)M.ntiles[0], tb, 0, s>>>(c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, psi,
+                                                                 c->ws.texp);
         note_launch((flosic_ctx*)c);
         k_hamiltonian_ix<<<(unsigned)M.ntiles[0], dim3(kTileX / 2, kTileY), kHSmem, s>>>(
-            c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, psi, vloc, vavg, texp, hpsi);
+            c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, psi, vloc, vavg, c->ws.texp, hpsi);
     } else
         k_hamiltonian64<<<(unsigned)M.ntiles[0], tb, 0, s>>>(c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, psi,
                                                               vloc, vavg, hpsi);

@@ -180,6 +180,7 @@ struct Workspace {
     double *z64, *p64b;              // multigrid PCG (FP64): z = M r, V-cycle scratch
     float *z32, *p32b;               // multigrid PCG (FP32)
     CgState cg;
+    int* texp;             // [level-0 tiles] largest exponent of the operand per tile (mixed Hamiltonian apply)
 };
 
 struct Multigrid {
