@@ -28,9 +28,9 @@ __constant__ double c_w64[kHalf + 1];   // this file's copy of the 12th-order we
 // the z-windows).  The two digits need 6 integer additions (three-operand) and
 // 2 multiply-adds per distance, against error-free sums and products of pairs.
 // A value is split once, when its plane arrives (IxStage); one barrier per
-// plane; the z-loop is unrolled 4 times (13 times, which keeps every window
-// slot in place, ran 30 % slower: the code no longer fits the instruction
-// cache).  128^3 x 64 orbitals with both potentials: 5.82 -> 2.32 ms, of which
+// plane.  With the z-loop unrolled 13 times, which keeps every window slot in
+// place, a third of the issue slots waited for instructions (2.7 -> 3.5 ms).
+// 128^3 x 64 orbitals with both potentials: 5.82 -> 2.24 ms, of which
 // k_tile_exp 0.15.
 // ---------------------------------------------------------------------------
 constexpr int kHSmem = kIxPts * 8 * kIxRing;

@@ -58,8 +58,10 @@ __device__ __forceinline__ ff ix_to_ff_b(long long I, float Lo) {
 }
 
 // z-windows in registers: the z-loop is unrolled kZU times, step u's window of
-// 13 planes in slots u .. u + 12, and moved down by kZU slots after the last.
-constexpr int kZU = 4, kQ = 2 * kHalf + kZU;
+// 13 planes in slots u .. u + 12, and moved down by kZU slots after the last
+// (twice: more spills at 128 registers; 13 times, which moves nothing, no longer
+// fits the instruction cache).
+constexpr int kZU = 2, kQ = 2 * kHalf + kZU;
 template <class Pt>
 __device__ __forceinline__ void ix_shift(Pt (&q)[kQ]) {
 #pragma unroll

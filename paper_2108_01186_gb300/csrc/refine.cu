@@ -177,18 +177,20 @@ __global__ void __launch_bounds__(256) k_residual12_ff(const BlkDesc* __restrict
 // of 2^(e-28) / 831600 in h^2 Delta_h d per point -- about 1e-14 of
 // max |d| / h^2, below the float-float sweep's error on smooth fields.
 // ---------------------------------------------------------------------------
-struct __align__(8) IxPt {
-    int h;     // rint(y)
-    float l;   // y - rint(y), or y itself when it is not finite
+// Two neighbouring points' parts, the low ones side by side for packed
+// two-lane additions.
+struct __align__(16) IxPair {
+    int h0, h1;      // rint(y) of either point
+    float2 l;        // y - rint(y)
 };
 
 // y = d 2^es (exact) split into hi + lo, for sums taken in unsigned (wrapping)
 // integers: a non-finite y carries inf / NaN in lo, so it reaches the
 // residual, and its saturated integer part only wraps the integer sum.
-__device__ __forceinline__ IxPt ix_split_w(float d, float s) {
-    const float y = d * s;
-    const float r = rintf(y);
-    return {__float2int_rn(r), y - r};
+__device__ __forceinline__ IxPair ix_split_w(float2 d, float s) {
+    const float y0 = d.x * s, y1 = d.y * s;
+    const float r0 = rintf(y0), r1 = rintf(y1);
+    return {__float2int_rn(r0), __float2int_rn(r1), make_float2(y0 - r0, y1 - r1)};
 }
 
 // Per orbital, max |d| over its grid (float bits in st.dmax, atomicMax on
@@ -234,45 +236,39 @@ __device__ __forceinline__ IxScale ix_scale(unsigned dmax, double h) {
             to_ff(d2ff(ldexp(1.0 / ((double)kW12Den * h * h), -es)))};
 }
 
-// The weighted sums (integer and float parts) of two neighbouring points:
-// pc the first one in the split plane of kPitch columns, q0 and q1 their
-// z-windows with plane z - 6 in slot u.
+// The weighted sums (integer and float parts) of a pair of points: pc its
+// entry in the split plane of kPitch pairs, q its z-window with plane z - 6 in
+// slot u.  The low parts of the two points run as packed two-lane operations
+// (the x-neighbours at odd distances are not pairs: two plain additions).
 template <int kPitch>
-__device__ __forceinline__ void ix_sums2(const IxPt* pc, const IxPt (&q0)[kQ], const IxPt (&q1)[kQ], int u,
-                                         long long& I0, long long& I1, float& L0, float& L1) {
+__device__ __forceinline__ void ix_sums2(const IxPair* pc, const IxPair (&q)[kQ], int u, long long& I0, long long& I1,
+                                         float2& Lo) {
     constexpr int kWc = (int)w12_centre3();
     constexpr int kW[kHalf + 1] = {kWc,           (int)w12_int(1), (int)w12_int(2), (int)w12_int(3),
                                    (int)w12_int(4), (int)w12_int(5), (int)w12_int(6)};
-    IxPt xw[2 * kHalf + 2];   // columns -6 .. 7 of the row, as 7 pairs
+    IxPair xw[kHalf + 1];   // columns -6 .. 7 of the row
 #pragma unroll
-    for (int k2 = 0; k2 < kHalf + 1; ++k2) {
-        const int4 v = *reinterpret_cast<const int4*>(pc - kHalf + 2 * k2);
-        xw[2 * k2] = {v.x, __int_as_float(v.y)};
-        xw[2 * k2 + 1] = {v.z, __int_as_float(v.w)};
-    }
-    const IxPt c0 = q0[u + kHalf], c1 = q1[u + kHalf];
-    I0 = (long long)kW[0] * c0.h;
-    I1 = (long long)kW[0] * c1.h;
-    L0 = (float)kW[0] * c0.l;
-    L1 = (float)kW[0] * c1.l;
+    for (int k2 = 0; k2 < kHalf + 1; ++k2) xw[k2] = pc[k2 - kHalf / 2];
+    auto xh = [&](int c) { return (unsigned)((c & 1) ? xw[c >> 1].h1 : xw[c >> 1].h0); };
+    auto xl = [&](int c) { return (c & 1) ? xw[c >> 1].l.y : xw[c >> 1].l.x; };
+    const IxPair c = q[u + kHalf];
+    I0 = (long long)kW[0] * c.h0;
+    I1 = (long long)kW[0] * c.h1;
+    Lo = __fmul2_rn(make_float2((float)kW[0], (float)kW[0]), c.l);
 #pragma unroll
     for (int m = 1; m <= kHalf; ++m) {
-        const int4 uu = *reinterpret_cast<const int4*>(pc - m * kPitch);   // rows -+ m
-        const int4 ww = *reinterpret_cast<const int4*>(pc + m * kPitch);
-        const IxPt a0 = q0[u + kHalf - m], b0 = q0[u + kHalf + m];
-        const IxPt a1 = q1[u + kHalf - m], b1 = q1[u + kHalf + m];
-        const unsigned h0 = (((unsigned)xw[kHalf - m].h + (unsigned)xw[kHalf + m].h) + ((unsigned)uu.x + (unsigned)ww.x)) +
-                            ((unsigned)a0.h + (unsigned)b0.h);
-        const unsigned h1 = (((unsigned)xw[kHalf + 1 - m].h + (unsigned)xw[kHalf + 1 + m].h) +
-                             ((unsigned)uu.z + (unsigned)ww.z)) + ((unsigned)a1.h + (unsigned)b1.h);
-        const float l0 = ((xw[kHalf - m].l + xw[kHalf + m].l) + (__int_as_float(uu.y) + __int_as_float(ww.y))) +
-                         (a0.l + b0.l);
-        const float l1 = ((xw[kHalf + 1 - m].l + xw[kHalf + 1 + m].l) + (__int_as_float(uu.w) + __int_as_float(ww.w))) +
-                         (a1.l + b1.l);
+        const IxPair uu = pc[-m * kPitch], ww = pc[m * kPitch];   // rows -+ m
+        const IxPair a = q[u + kHalf - m], b = q[u + kHalf + m];
+        const unsigned h0 = ((xh(kHalf - m) + xh(kHalf + m)) + ((unsigned)uu.h0 + (unsigned)ww.h0)) +
+                            ((unsigned)a.h0 + (unsigned)b.h0);
+        const unsigned h1 = ((xh(kHalf + 1 - m) + xh(kHalf + 1 + m)) + ((unsigned)uu.h1 + (unsigned)ww.h1)) +
+                            ((unsigned)a.h1 + (unsigned)b.h1);
+        const float2 x2 = (m & 1) ? make_float2(xl(kHalf - m) + xl(kHalf + m), xl(kHalf + 1 - m) + xl(kHalf + 1 + m))
+                                  : __fadd2_rn(xw[(kHalf - m) >> 1].l, xw[(kHalf + m) >> 1].l);
+        const float2 l = __fadd2_rn(__fadd2_rn(x2, __fadd2_rn(uu.l, ww.l)), __fadd2_rn(a.l, b.l));
         I0 += (long long)kW[m] * (int)h0;
         I1 += (long long)kW[m] * (int)h1;
-        L0 = fmaf((float)kW[m], l0, L0);
-        L1 = fmaf((float)kW[m], l1, L1);
+        Lo = __ffma2_rn(make_float2((float)kW[m], (float)kW[m]), l, Lo);
     }
 }
 
@@ -280,7 +276,9 @@ __device__ __forceinline__ void ix_sums2(const IxPt* pc, const IxPt (&q0)[kQ], c
 __device__ __forceinline__ ff ix_update(long long I, float Lo, ff cf, float2 r) {
     return ff_add(to_ff(r), ff_mul(ix_to_ff_b(I, Lo), cf));
 }
-__device__ __forceinline__ float ix_centre(IxPt c, float is) { return (__int2float_rn(c.h) + c.l) * is; }
+__device__ __forceinline__ float2 ix_centre(IxPair c, float is) {
+    return make_float2((__int2float_rn(c.h0) + c.l.x) * is, (__int2float_rn(c.h1) + c.l.y) * is);
+}
 __device__ __forceinline__ ff ix_add(float2 x, float d) {   // x + d
     const ff s = ff_two_sum(x.x, d);
     return ff_quick(s.h, s.l + x.y);
@@ -296,16 +294,20 @@ __device__ __forceinline__ ff ix_add(float2 x, float d) {   // x + d
 // start from d = 0.  kXZ: the first update after a cold start that stored no
 // x (x = 0, not read).
 //
-// This form has its operands staged by the copy engine (blocks whose rows and offset are 16-byte aligned and that have no periodic
-// direction: the zero fill of the copies is the zero ghost value).  A ring
-// of kURing stages runs ahead of the z-march, each holding the plane z of d
-// with its halo (48 x 28: x0 - 8 keeps the copy 16-byte aligned), d at
-// plane z + 6 (32 x 16, the head of the register z-queues) and r and x at
-// plane z (32 x 16 pairs).  Each plane's d is split once into shared memory
+// This form has its operands staged by the copy engine (blocks whose rows and
+// offset are 16-byte aligned and that have no periodic direction: the zero fill
+// of the copies is the zero ghost value).  A ring of kURing stages runs ahead of
+// the z-march, each holding the plane z of d with its halo (48 x 28: x0 - 8
+// keeps the copy 16-byte aligned), d at plane z + 6 (32 x 16, the head of the
+// register z-queues) and r and x at plane z (32 x 16 pairs).  Each plane's d is
+// split once into shared memory
 // (hi, lo; two buffers, so one barrier per plane serves both the split plane
-// and the stage of the plane before); a thread owns the two points (x0 + 2 tx + a, y0 + ty), reads
-// their x-window (14 values) and y-windows as 16-byte pairs and keeps their
-// z-windows in registers.
+// and the stage of the plane before); a thread owns the two points (x0 + 2 tx +
+// a, y0 + ty), reads their x-window (14 values) and y-windows as 16-byte pairs
+// and keeps their z-windows in registers.
+// What bounds it: instruction issue and shared-memory traffic.  With the parts
+// of a point pair side by side (16-byte splits and stores, packed low-part sums)
+// Poisson solves of 128^3 x 64 take 6.93 -> 6.71 ms, 192^3 x 24 8.94 -> 8.66.
 constexpr int kUX = 48;                              // staged width: x0 - 8 .. x0 + 39
 constexpr int kUY = kTileY + 2 * kHalf;              // 28: y0 - 6 .. y0 + 21
 constexpr int kUPlane = kUX * kUY;                   // floats of the halo plane
@@ -315,7 +317,7 @@ constexpr int kURing = 5;
 constexpr unsigned kUStageBytes = 4u * kUStage;
 
 // the stages, two split planes (one barrier per plane), the stages' mbarriers
-size_t update_tma_smem() { return 4 * (size_t)kURing * kUStage + 2 * sizeof(IxPt) * kUPlane + 8 * kURing + 128; }
+size_t update_tma_smem() { return 4 * (size_t)kURing * kUStage + sizeof(IxPair) * kUPlane + 8 * kURing + 128; }
 
 template <bool kXZ>
 __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restrict__ blk, const LvlDesc* __restrict__ L,
@@ -328,8 +330,8 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
     extern __shared__ __align__(128) unsigned char us_raw[];
     unsigned char* smem = us_raw + ((128 - (tc_smem_addr(us_raw) & 127)) & 127);
     float* ring = reinterpret_cast<float*>(smem);
-    IxPt* spb = reinterpret_cast<IxPt*>(smem + 4 * (size_t)kURing * kUStage);   // two split planes
-    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 4 * (size_t)kURing * kUStage + 2 * sizeof(IxPt) * kUPlane);
+    IxPair* spb = reinterpret_cast<IxPair*>(smem + 4 * (size_t)kURing * kUStage);   // two split planes
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 4 * (size_t)kURing * kUStage + sizeof(IxPair) * kUPlane);
     __shared__ double scratch[32];
     const TilePos P = tile_pos(blk, L, tiles, orb_blk, blockIdx.x);
     if (!st.oactive[P.o] || !L[P.b].utma) return;
@@ -369,17 +371,16 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
     const long long dsz = (long long)B.p[0] * B.p[1];
     const long long dcol = B.poff + (long long)oi * B.Gp + (long long)gy * B.p[0] + gx;
     // z-windows of the two points: plane z - 6 + j of step k0 + u in slot u + j
-    IxPt q0[kQ], q1[kQ];
+    IxPair q[kQ];
 #pragma unroll
     for (int j = 0; j < 2 * kHalf; ++j) {
         const int zz = P.z0 - kHalf + j;
         float2 v = make_float2(0.f, 0.f);
         if (in && zz >= 0 && zz < D.nz) v = *reinterpret_cast<const float2*>(d32 + zz * dsz + dcol);
-        q0[j] = ix_split_w(v.x, sc);
-        q1[j] = ix_split_w(v.y, sc);
+        q[j] = ix_split_w(v, sc);
     }
     float rrf = 0.f;
-    const int ly = ty + kHalf, cx = 2 * tx + 8;       // the points' row and first column in the staged plane
+    const int pc = (ty + kHalf) * (kUX / 2) + tx + 4;   // the points' pair in the staged plane
     for (int k0 = 0; k0 < nzt; k0 += kZU) {
 #pragma unroll
         for (int u = 0; u < kZU; ++u) {
@@ -387,13 +388,10 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
             if (k >= nzt) break;
             if (!tc_mbar_wait(bar + (k % kURing), (uint32_t)((k / kURing) & 1))) atomicOr(status + 3, 8);
             const float* sg = ring + (size_t)(k % kURing) * kUStage;
-            IxPt* const sp = spb + (k & 1) * kUPlane;
-            for (int e = tid; e < kUPlane; e += 256) sp[e] = ix_split_w(sg[e], sc);
-            {
-                const float2 hv = *reinterpret_cast<const float2*>(sg + kUPlane + ty * kTileX + 2 * tx);
-                q0[u + 2 * kHalf] = ix_split_w(hv.x, sc);
-                q1[u + 2 * kHalf] = ix_split_w(hv.y, sc);
-            }
+            IxPair* const sp = spb + (k & 1) * (kUPlane / 2);
+            for (int e = tid; e < kUPlane / 2; e += 256) sp[e] = ix_split_w(reinterpret_cast<const float2*>(sg)[e], sc);
+            q[u + 2 * kHalf] =
+                ix_split_w(*reinterpret_cast<const float2*>(sg + kUPlane + ty * kTileX + 2 * tx), sc);
             // the split plane is written, and every thread has finished plane k - 1: its
             // stage takes plane k - 1 + kURing (the other split plane is free for plane k + 1)
             __syncthreads();
@@ -402,16 +400,16 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
                 issue(k - 1 + kURing);
             }
             long long I0, I1;
-            float L0, L1;
-            ix_sums2<kUX>(sp + ly * kUX + cx, q0, q1, u, I0, I1, L0, L1);
+            float2 Lo;
+            ix_sums2<kUX / 2>(sp + pc, q, u, I0, I1, Lo);
             if (in) {
                 const float4 rv = *reinterpret_cast<const float4*>(sg + kUPlane + kUCtr + ty * 2 * kTileX + 4 * tx);
                 const float4 xv = xz ? make_float4(0.f, 0.f, 0.f, 0.f)
                                      : *reinterpret_cast<const float4*>(sg + kUPlane + 3 * kUCtr + ty * 2 * kTileX + 4 * tx);
                 const long long g = P.base + (P.z0 + k) * sz + col;
-                const ff rn[2] = {ix_update(I0, L0, cf, make_float2(rv.x, rv.y)), ix_update(I1, L1, cf, make_float2(rv.z, rv.w))};
-                const ff xn[2] = {ix_add(make_float2(xv.x, xv.y), ix_centre(q0[u + kHalf], is)),
-                                  ix_add(make_float2(xv.z, xv.w), ix_centre(q1[u + kHalf], is))};
+                const ff rn[2] = {ix_update(I0, Lo.x, cf, make_float2(rv.x, rv.y)), ix_update(I1, Lo.y, cf, make_float2(rv.z, rv.w))};
+                const float2 dc = ix_centre(q[u + kHalf], is);
+                const ff xn[2] = {ix_add(make_float2(xv.x, xv.y), dc.x), ix_add(make_float2(xv.z, xv.w), dc.y)};
                 rrf += rn[0].h * rn[0].h;
                 rrf += rn[1].h * rn[1].h;
                 *reinterpret_cast<float4*>(r + g) = make_float4(rn[0].h, rn[0].l, rn[1].h, rn[1].l);
@@ -419,8 +417,7 @@ __global__ void __launch_bounds__(256, 2) k_update12_tma(const BlkDesc* __restri
                 *reinterpret_cast<float2*>(r32 + (P.z0 + k) * dsz + dcol) = make_float2(rn[0].h, rn[1].h);
             }
         }
-        ix_shift(q0);
-        ix_shift(q1);
+        ix_shift(q);
     }
     if (tile_arrive(rrf, st.part, blockIdx.x, st.count + P.o, D.ntile, scratch)) {
         const double sum = tile_gather(st.part, P.first, D.ntile, scratch);
@@ -454,7 +451,7 @@ __global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restric
                                                         double* __restrict__ V, float* __restrict__ r32, double tol2,
                                                         double inner_tol2, int max_iter, CgState st) {
     extern __shared__ __align__(16) unsigned char uc_raw[];
-    IxPt* const ring = reinterpret_cast<IxPt*>(uc_raw);
+    IxPair* const ring = reinterpret_cast<IxPair*>(uc_raw);
     float2* const rx = reinterpret_cast<float2*>(uc_raw + kCOffRx);   // [2][r pairs, V][kUCtr]
     __shared__ double scratch[32];
     const TilePos P = tile_pos(blk, L, tiles, orb_blk, blockIdx.x);
@@ -480,16 +477,14 @@ __global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restric
         const float* pl = d32 + db + (okz ? z * dsz : 0);
 #pragma unroll
         for (int j = 0; j < kIxU; ++j)
-            if (sg.wants(j, k < nzt)) sg.copy(j, ring + slot * kIxPts + 2 * (tid + j * 256), pl, okz, vec, nx);
+            if (sg.wants(j, k < nzt)) sg.copy(j, ring + slot * kIxPairs + tid + j * 256, pl, okz, vec, nx);
     };
     auto split = [&](int k, int slot, float sc) {
 #pragma unroll
         for (int j = 0; j < kIxU; ++j)
             if (sg.wants(j, k < nzt)) {
-                IxPt* const at = ring + slot * kIxPts + 2 * (tid + j * 256);
-                const float2 v = *reinterpret_cast<const float2*>(at);
-                const IxPt a = ix_split_w(v.x, sc), b = ix_split_w(v.y, sc);
-                *reinterpret_cast<int4*>(at) = make_int4(a.h, __float_as_int(a.l), b.h, __float_as_int(b.l));
+                IxPair* const at = ring + slot * kIxPairs + tid + j * 256;
+                *at = ix_split_w(*reinterpret_cast<const float2*>(at), sc);
             }
     };
     // r and V of plane z0 + k: rows of 32 points per warp
@@ -517,28 +512,24 @@ __global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restric
     const int gx = P.x0 + 2 * tx, gy = P.y0 + ty;
     const bool in0 = gx < nx && gy < ny, in1 = gx + 1 < nx && gy < ny;
     const long long col = gy * sy + gx, dcol = db + (long long)gy * dpx + gx;
-    const int ctr = (ty + kHalf) * kPX + 2 * tx + kHalf;   // the first point in a staged plane
+    const int ctr = (ty + kHalf) * (kPX / 2) + tx + kHalf / 2;   // the pair in a staged plane
     __syncthreads();
     const float sc = s_scale.sc, is = s_scale.is;
     const ff cf = s_scale.cf;
-    IxPt q0[kQ], q1[kQ];   // z-windows: step k0 + u's in slots u .. u + 12
+    IxPair q[kQ];   // z-windows: step k0 + u's in slots u .. u + 12
 #pragma unroll
     for (int j = 0; j < kHalf; ++j) {   // planes z0 - 6 .. z0 - 1 straight from memory
         int z = P.z0 - kHalf + j;
         if (per & 4) z = wrap_coord(z, nz);
         const float* pl = d32 + z * dsz + dcol;
-        q0[j] = ix_split_w(z >= 0 && z < nz && in0 ? pl[0] : 0.f, sc);
-        q1[j] = ix_split_w(z >= 0 && z < nz && in1 ? pl[1] : 0.f, sc);
+        const bool okz = z >= 0 && z < nz;
+        q[j] = ix_split_w(make_float2(okz && in0 ? pl[0] : 0.f, okz && in1 ? pl[1] : 0.f), sc);
     }
     asm volatile("cp.async.wait_group 2;" ::: "memory");
     for (int k = 0; k < kHalf; ++k) split(k, k, sc);
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kHalf; ++k) {
-        const int4 hv = *reinterpret_cast<const int4*>(ring + k * kIxPts + ctr);
-        q0[kHalf + k] = {hv.x, __int_as_float(hv.y)};
-        q1[kHalf + k] = {hv.z, __int_as_float(hv.w)};
-    }
+    for (int k = 0; k < kHalf; ++k) q[kHalf + k] = ring[k * kIxPairs + ctr];
     float rrf = 0.f;
     int slot = 0;   // of plane z0 + k
     for (int k0 = 0; k0 < nzt; k0 += kZU) {
@@ -558,20 +549,17 @@ __global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restric
             __syncthreads();
             if (k + 1 < nzt) copy_rx(k + 1);
             cp_async_commit();
-            {
-                const int4 hv = *reinterpret_cast<const int4*>(ring + hslot * kIxPts + ctr);
-                q0[u + 2 * kHalf] = {hv.x, __int_as_float(hv.y)};
-                q1[u + 2 * kHalf] = {hv.z, __int_as_float(hv.w)};
-            }
-            const IxPt* const pc = ring + slot * kIxPts + ctr;
+            q[u + 2 * kHalf] = ring[hslot * kIxPairs + ctr];
+            const IxPair* const pc = ring + slot * kIxPairs + ctr;
             slot = ix_slot(slot, 1);
             long long I0, I1;
-            float L0, L1;
-            ix_sums2<kPX>(pc, q0, q1, u, I0, I1, L0, L1);
+            float2 Lo;
+            ix_sums2<kPX / 2>(pc, q, u, I0, I1, Lo);
             const float2* const st2 = rx + (k & 1) * 2 * kUCtr + ty * kTileX + 2 * tx;
             const float4 rv = *reinterpret_cast<const float4*>(st2);
-            const ff rn[2] = {ix_update(I0, L0, cf, make_float2(rv.x, rv.y)), ix_update(I1, L1, cf, make_float2(rv.z, rv.w))};
-            double2 vn = make_double2(f2d(ix_centre(q0[u + kHalf], is)), f2d(ix_centre(q1[u + kHalf], is)));
+            const ff rn[2] = {ix_update(I0, Lo.x, cf, make_float2(rv.x, rv.y)), ix_update(I1, Lo.y, cf, make_float2(rv.z, rv.w))};
+            const float2 dc = ix_centre(q[u + kHalf], is);
+            double2 vn = make_double2(f2d(dc.x), f2d(dc.y));
             if (!kXZ) {
                 const double2 vo = *reinterpret_cast<const double2*>(st2 + kUCtr);
                 vn.x += vo.x;
@@ -592,8 +580,7 @@ __global__ void __launch_bounds__(256, 2) k_update12_cp(const BlkDesc* __restric
                 rrf += rn[1].h * rn[1].h;
             }
         }
-        ix_shift(q0);
-        ix_shift(q1);
+        ix_shift(q);
     }
     if (tile_arrive(rrf, st.part, blockIdx.x, st.count + P.o, D.ntile, scratch)) {
         const double sum = tile_gather(st.part, P.first, D.ntile, scratch);
