@@ -441,19 +441,25 @@ __global__ void __launch_bounds__(256, RM <= 2 ? 2 : 1) k_contract_f(const BlkDe
     }
 }
 
-// out[e] = sum_kp part[kp][e] in a fixed order: a CTA takes 8 elements, 32
-// threads each (one thread per element waited for one load after the other:
-// 608 parts of 25 elements 94 us, now 7)
-__global__ void __launch_bounds__(256) k_sum_parts(const double* __restrict__ part, int kparts, long long n,
-                                                   double* __restrict__ out) {
-    const long long e = (long long)blockIdx.x * 8 + (threadIdx.x & 7);
+// out[e] = sum_kp part[kp][e] in order of kp.  One warp per 32 elements and 16
+// loads in flight: the plain loop waited for one load after the other (608
+// parts of 25 elements 94 us).  The order stays: in the mixed path a last bit of
+// these sums decides roundings to float32 further on.
+__global__ void __launch_bounds__(32) k_sum_parts(const double* __restrict__ part, int kparts, long long n,
+                                                  double* __restrict__ out) {
+    const long long e = (long long)blockIdx.x * 32 + threadIdx.x;
+    if (e >= n) return;
     double s = 0.0;
-    if (e < n) {
-#pragma unroll 8
-        for (int k = threadIdx.x >> 3; k < kparts; k += 32) s += part[(long long)k * n + e];
+    int k = 0;
+    for (; k + 16 <= kparts; k += 16) {
+        double v[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = part[(long long)(k + j) * n + e];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) s += v[j];
     }
-    s = sum_of_8(s);
-    if (threadIdx.x < 8 && e < n) out[e] = s;
+    for (; k < kparts; ++k) s += part[(long long)k * n + e];
+    out[e] = s;
 }
 
 static int max_block_n(const flosic_ctx* c) {
@@ -486,7 +492,7 @@ static void contract(const flosic_ctx* c, LA la, LB lb, double* out, cudaStream_
         else k_contract<8, double><<<grid, 256, 0, s>>>(c->d_blk, kparts, la, lb, part, c->mat_elems);
     }
     note_launch(c);
-    k_sum_parts<<<(unsigned)((c->mat_elems + 7) / 8), 256, 0, s>>>(part, kparts, c->mat_elems, out); note_launch(c);
+    k_sum_parts<<<(unsigned)((c->mat_elems + 31) / 32), 32, 0, s>>>(part, kparts, c->mat_elems, out); note_launch(c);
 }
 
 // Raw Gram psi psi^T per block: tensor cores (split-BF16) in mixed precision,

@@ -418,27 +418,30 @@ __global__ void __launch_bounds__(288, 1) k_gram_async(const BlkDesc* __restrict
 }
 
 // M[block][e] = sum over the block's partials (pk per chunk, pk = the
-// launch's sub-chunk count, set by its widest block) in float64: a CTA takes 8
-// elements, 32 threads each, whose sums are added in a fixed order.  The
-// conversions are integer operations, so the float64 pipe has one addition per
-// partial, and 8 elements a CTA spread them over all SMs (32 elements and
-// hardware conversions: 95 us for the 2 x 4096 partials of 32 x 32 at 128^3, now
-// 79).
+// launch's sub-chunk count, set by its widest block) in float64: a CTA takes
+// 32 elements; its 8 warps sum every 8th partial each, and the 8 sums are
+// added in a fixed order.
 __global__ void __launch_bounds__(256) k_gram_sum(const BlkDesc* __restrict__ blk, const float* __restrict__ part,
                                                   const long long* __restrict__ part_off, double* __restrict__ M,
                                                   int pk) {
+    __shared__ double red[8][32];
     const BlkDesc& B = blk[blockIdx.y];
     const int NN2 = B.N * B.N;
-    const int e = blockIdx.x * 8 + (threadIdx.x & 7);
+    const int e = blockIdx.x * 32 + (threadIdx.x & 31), w = threadIdx.x >> 5;
     const long long nparts = ((B.G + kGChunk - 1) / kGChunk) * pk;
     double s = 0.0;
     if (e < NN2) {
         const float* p = part + part_off[blockIdx.y] + e;
 #pragma unroll 8
-        for (long long q = threadIdx.x >> 3; q < nparts; q += 32) s += f2d(p[q * NN2]);
+        for (long long q = w; q < nparts; q += 8) s += (double)p[q * NN2];
     }
-    s = sum_of_8(s);
-    if (threadIdx.x < 8 && e < NN2) M[B.moff + e] = s;
+    red[w][threadIdx.x & 31] = s;
+    __syncthreads();
+    if (w == 0 && e < NN2) {
+        double t = 0.0;
+        for (int k = 0; k < 8; ++k) t += red[k][threadIdx.x];
+        M[B.moff + e] = t;
+    }
 }
 
 // sub-chunk partials per chunk of every block: set by the widest block, whose
@@ -517,7 +520,7 @@ void launch_gram_tc(const flosic_ctx* c, const double* psi, cudaStream_t s) {
         cudaEventRecord(cm->ov_ev[2 * cm->ov_used + 1], s);
         ++cm->ov_used;
     }
-    const dim3 g2((unsigned)((nmax * nmax + 7) / 8), (unsigned)c->nblk);
+    const dim3 g2((unsigned)((nmax * nmax + 31) / 32), (unsigned)c->nblk);
     k_gram_sum<<<g2, 256, 0, s>>>(c->d_blk, part, off, c->ws.M, gram_launch_pack(c));
     note_launch((flosic_ctx*)c);
 }

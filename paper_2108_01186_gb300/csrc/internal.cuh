@@ -596,20 +596,6 @@ __device__ __forceinline__ ff warp_sum(ff v) {
     return v;
 }
 
-// Sums the partials of 8 elements (element tid & 7) over the 32 threads of a
-// CTA of 256 that hold each, in a fixed order; the totals come back in threads 0 .. 7.
-__device__ __forceinline__ double sum_of_8(double v) {
-    __shared__ double red8[8][8];
-    v += __shfl_xor_sync(0xffffffffu, v, 8);
-    v += __shfl_xor_sync(0xffffffffu, v, 16);
-    if ((threadIdx.x & 31) < 8) red8[threadIdx.x >> 5][threadIdx.x & 7] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x < 8)
-        for (int w = 0; w < 8; ++w) t += red8[w][threadIdx.x];
-    return t;
-}
-
 // index of point (x, y, z) of orbital i of block B in the Kronecker solver's padded arrays
 __device__ __forceinline__ long long pad_index(const BlkDesc& B, int i, int x, int y, int z) {
     return B.poff + (long long)i * B.Gp + ((long long)z * B.p[1] + y) * B.p[0] + x;
