@@ -640,14 +640,8 @@ def time_uneven(dev, stream, solver, steps=3):
     from paper_2108_01186_gb300.flosic import Context
     systems = synth.make_uneven_batch(nsys=64, seed_base=2000)
     norb = sum(sum(x.norb) for x in systems)
-    # blocks on the tensor-core transforms: sides multiples of 8 (<= 128) and a
-    # 16-byte-aligned offset in the packed orbital arrays
-    n_tc, off = 0, 0
-    for x in systems:
-        if x.n % 8 == 0 and x.n <= 128 and off % 4 == 0:
-            n_tc += 1
-        off += x.norb[0] * x.G
     ctx = Context(systems, precision=1, cg_tol=CG_TOL, preconditioner=1, solver=solver)
+    n_tc = sum(bool(p["tensor_core_transforms"]) for p in ctx.block_paths())
     psi = torch.tensor(np.concatenate([p.ravel() for x in systems for p in x.psi]), device=dev)
     fods = torch.tensor(np.concatenate([f.ravel() for x in systems for f in x.fods]), device=dev)
     del systems
