@@ -331,7 +331,8 @@ __device__ __forceinline__ void tc_issue_unit(bool full, int ksteps, uint32_t dm
 // for the units of the tile two before it.  The converters fold the next
 // tile's rows into registers while the current tile's MMAs run.  Every wait
 // sleeps on its mbarrier, gives up after about two seconds or as soon as
-// another warp has given up (s_abort), and the decision is warp-uniform.
+// another warp has given up (s_abort), and the lanes vote on the outcome
+// (tc_mbar_warp_wait), so a warp leaves its loop as a whole.
 template <int HP>
 __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long long total) {
     using S = TcShape<HP>;
@@ -389,8 +390,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
         int ksteps = 0, nch = 0, cb = -1;
         uint32_t sl = 0, use = 0;       // ring slot of the next unit, and how often it was used
         for (int t = 0;; ++t) {
-            bool ok = tc_mbar_sleep_or_abort(&bar_conv[0], (uint32_t)(t & 1), &s_abort);
-            if (!__all_sync(0xffffffffu, ok)) { s_abort = 1; break; }
+            bool ok = tc_mbar_warp_wait(&bar_conv[0], (uint32_t)(t & 1), &s_abort);
+            if (!ok) { s_abort = 1; break; }
             const TcTile cur = s_tile[t % kTcInfo];   // (written before the copies this tile's converters waited for)
             const int tb = (int)tc_uniform((uint32_t)cur.b);
             if (tb < 0) break;
@@ -404,11 +405,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
             // unit u of the tile: half u / nch, chunk u mod nch (kHalves), or chunk u / 2, half u mod 2
             for (int u = 0, h = 0, c = 0; u < 2 * nch; ++u) {
                 if (S::kHalves ? u == nch : u == 0) {   // the second half's splits
-                    ok = tc_mbar_sleep_or_abort(&bar_conv[1], (uint32_t)(t & 1), &s_abort);
+                    ok = tc_mbar_warp_wait(&bar_conv[1], (uint32_t)(t & 1), &s_abort);
                 }
                 // the unit that last used this slot has been read
-                if (use > 0) ok = ok && tc_mbar_sleep_or_abort(&bar_free[sl], (use - 1) & 1, &s_abort);
-                ok = __all_sync(0xffffffffu, ok);
+                if (use > 0) ok = ok && tc_mbar_warp_wait(&bar_free[sl], (use - 1) & 1, &s_abort);
                 if (!ok) break;
                 tc_fence_after();
                 tc_issue_unit<HP>(a.full != 0, ksteps, t0 + sl * (2 * kTcUnit), t0 + S::kColA + (uint32_t)(h * 3 * (HP / 2)),
@@ -447,8 +447,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
                 tc_blk_load(kc, a.blk, nt.b, a.axis);
                 const int nbox = (kc.p + 31) >> 5;
                 while (used + nbox > S::kBoxes && ok) {   // the oldest staged tile has been read
-                    ok = tc_mbar_sleep_or_abort(&bar_raw[tail % kTcInfo], (uint32_t)((tail / kTcInfo) & 1), &s_abort);
-                    ok = __all_sync(0xffffffffu, ok);
+                    ok = tc_mbar_warp_wait(&bar_raw[tail % kTcInfo], (uint32_t)((tail / kTcInfo) & 1), &s_abort);
                     used -= s_nbox[tail % kTcInfo];
                     ++tail;
                 }
@@ -491,12 +490,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
         uint32_t box_uses = 0;                           // parity bit per ring slot of its next completion
         TcBlk kb;
         for (int t = 0;; ++t) {
-            bool ok = tc_mbar_sleep_or_abort(&bar_info[t % kTcInfo], (uint32_t)((t / kTcInfo) & 1), &s_abort);
-            if (!__all_sync(0xffffffffu, ok)) { s_abort = 1; break; }
+            bool ok = tc_mbar_warp_wait(&bar_info[t % kTcInfo], (uint32_t)((t / kTcInfo) & 1), &s_abort);
+            if (!ok) { s_abort = 1; break; }
             const int cb = s_tile[t % kTcInfo].b;
             if (cb < 0) {   // the MMA warp learns it through bar_conv (after it has seen the last tile's)
-                ok = t < 1 || tc_mbar_sleep_or_abort(&bar_half[1], (uint32_t)((t - 1) & 1), &s_abort);
-                if (__all_sync(0xffffffffu, ok) && lane == 0) tc_mbar_arrive(&bar_conv[0]);
+                ok = t < 1 || tc_mbar_warp_wait(&bar_half[1], (uint32_t)((t - 1) & 1), &s_abort);
+                if (ok && lane == 0) tc_mbar_arrive(&bar_conv[0]);
                 break;
             }
             tc_blk_load(kb, a.blk, cb, a.axis);
@@ -504,10 +503,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
             const int nbox = (kb.p + 31) >> 5;
             for (int bx = 0; bx < nbox && ok; ++bx) {
                 const int sl = box0 + bx >= S::kBoxes ? box0 + bx - S::kBoxes : box0 + bx;
-                ok = tc_mbar_sleep_or_abort(&bar_tma[sl], (box_uses >> sl) & 1u, &s_abort);
+                ok = tc_mbar_warp_wait(&bar_tma[sl], (box_uses >> sl) & 1u, &s_abort);
                 box_uses ^= 1u << sl;
             }
-            if (!__all_sync(0xffffffffu, ok)) { s_abort = 1; break; }
+            if (!ok) { s_abort = 1; break; }
             const int k16 = (ns + 15) & ~15;             // K values the MMAs read
             // the first groups folded into registers while the last tile's MMAs run
             float e[S::kPre][8], o[S::kPre][8];
@@ -523,8 +522,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
             // the last tile's MMAs have read the (first half's) operand splits; new
             // matrices wait for all of them
             const bool new_b = cb != loaded_b;
-            if (t >= 1) ok = tc_mbar_sleep_or_abort(&bar_half[S::kHalves && !new_b ? 0 : 1], (uint32_t)((t - 1) & 1), &s_abort);
-            if (!__all_sync(0xffffffffu, ok)) { s_abort = 1; break; }
+            if (t >= 1) ok = tc_mbar_warp_wait(&bar_half[S::kHalves && !new_b ? 0 : 1], (uint32_t)((t - 1) & 1), &s_abort);
+            if (!ok) { s_abort = 1; break; }
             tc_fence_after();
             if (new_b) {   // this block's matrices: the rows and K values in use
                 const uint16_t* src = a.mat + kb.kt + (a.inverse ? 6 * S::kMatElems : 0);
@@ -542,8 +541,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     if (h == 1 && t >= 1) {
-                        ok = tc_mbar_sleep_or_abort(&bar_half[1], (uint32_t)((t - 1) & 1), &s_abort);
-                        if (!__all_sync(0xffffffffu, ok)) { s_abort = 1; break; }
+                        ok = tc_mbar_warp_wait(&bar_half[1], (uint32_t)((t - 1) & 1), &s_abort);
+                        if (!ok) { s_abort = 1; break; }
                         tc_fence_after();
                     }
 #pragma unroll
@@ -601,8 +600,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
         TcBlk kb;
         bool ok = true;
         for (int t = 0; ok; ++t) {
-            ok = tc_mbar_sleep_or_abort(&bar_info[t % kTcInfo], (uint32_t)((t / kTcInfo) & 1), &s_abort);
-            if (!__all_sync(0xffffffffu, ok)) { s_abort = 1; break; }
+            ok = tc_mbar_warp_wait(&bar_info[t % kTcInfo], (uint32_t)((t / kTcInfo) & 1), &s_abort);
+            if (!ok) { s_abort = 1; break; }
             const TcTile cur = s_tile[t % kTcInfo];
             if (cur.b < 0) break;
             tc_blk_load(kb, a.blk, cur.b, a.axis);
@@ -633,9 +632,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
             for (int c = 0; c < nch; ++c) {
                 const uint32_t ue = U + (S::kHalves ? c : 2 * c), uo = U + (S::kHalves ? nch + c : 2 * c + 1);
                 const uint32_t s0 = ue % S::kUnits, s1 = uo % S::kUnits;
-                ok = tc_mbar_sleep_or_abort(&bar_full[s0], (ue / S::kUnits) & 1, &s_abort) &&
-                     tc_mbar_sleep_or_abort(&bar_full[s1], (uo / S::kUnits) & 1, &s_abort);
-                ok = __all_sync(0xffffffffu, ok);
+                ok = tc_mbar_warp_wait(&bar_full[s0], (ue / S::kUnits) & 1, &s_abort) &&
+                     tc_mbar_warp_wait(&bar_full[s1], (uo / S::kUnits) & 1, &s_abort);
                 if (!ok) { s_abort = 1; break; }
                 tc_fence_after();
                 const uint32_t te = tr + s0 * (2 * kTcUnit), to = tr + s1 * (2 * kTcUnit);

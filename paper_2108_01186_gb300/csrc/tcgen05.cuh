@@ -229,6 +229,14 @@ __device__ __forceinline__ bool tc_mbar_sleep_or_abort(uint64_t* bar, uint32_t p
     return false;
 }
 
+// The same for a converged warp: true if every lane saw the phase complete.  The
+// lanes poll on their own and may disagree near the limit or when *abort changes;
+// a warp whose code has collective operations ahead must branch on the vote, or
+// some lanes would wait for the others at the next one, outside any limit.
+__device__ __forceinline__ bool tc_mbar_warp_wait(uint64_t* bar, uint32_t parity, const volatile int* abort) {
+    return __all_sync(0xffffffffu, tc_mbar_sleep_or_abort(bar, parity, abort));
+}
+
 // named barrier over `count` threads (a multiple of 32) of the CTA
 __device__ __forceinline__ void tc_named_sync(int id, int count) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
