@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
     __shared__ __align__(16) float s_lam[4][S::kLam];
     __shared__ uint32_t tmem_base;
     __shared__ volatile int s_abort;
-    __shared__ int s_tma_issued[S::kBoxes], s_mma_issued;
+    __shared__ int s_tma_issued[S::kBoxes], s_units;   // copies per ring slot, units committed
     const int tid = threadIdx.x, warp = (int)tc_uniform((uint32_t)tid >> 5), lane = tid & 31;
     const long long per_cta = (total + gridDim.x - 1) / gridDim.x;
     const long long it0 = (long long)blockIdx.x * per_cta;
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
             tc_mbar_init(&bar_half[h], 1);
         }
         s_abort = 0;
-        s_mma_issued = 0;
+        s_units = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tmem_alloc(&tmem_base, kTcCols);
@@ -415,6 +415,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
                                   b0 + (uint32_t)(h * 3 * S::kBTile), c, el);
                 if (el) {
                     umma_commit(&bar_full[sl]);
+                    ++s_units;
                     if (u == 2 * nch - 1 || (S::kHalves && u == nch - 1)) umma_commit(&bar_half[u == 2 * nch - 1 ? 1 : 0]);
                 }
                 __syncwarp();
@@ -430,7 +431,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
                 }
             }
             if (!ok) { s_abort = 1; break; }
-            if (el) ++s_mma_issued;
         }
     } else if (warp == kTcThreads / 32 - 1) {
         // ---- the tile list and the copies (one elected lane issues) -------------
@@ -737,7 +737,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_kron_tc(KronTcArgs a, long lo
         // let the copies and the MMAs this CTA has in flight finish (bounded)
         for (int b = 0; b < S::kBoxes; ++b)
             if (s_tma_issued[b] > 0) tc_mbar_wait(&bar_tma[b], (uint32_t)((s_tma_issued[b] - 1) & 1));
-        if (s_mma_issued > 0) tc_mbar_wait(&bar_half[1], (uint32_t)((s_mma_issued - 1) & 1));
+        // (a commit covers every MMA before it, so the last unit's covers all, also in mid-tile)
+        const TcLastCommit lc = tc_last_commit(s_units, S::kUnits);
+        if (lc.slot >= 0) tc_mbar_wait(&bar_full[lc.slot], lc.parity);
     }
     __syncthreads();
     if (warp == 0) {

@@ -114,6 +114,21 @@ __device__ __forceinline__ uint32_t tc_elect() {
 // reduction's result is a uniform register; a shuffle's is not).
 __device__ __forceinline__ uint32_t tc_uniform(uint32_t v) { return __reduce_or_sync(0xffffffffu, v); }
 
+// The last of `count` commits made in turn to the mbarriers of a ring of `ring`
+// slots (one commit per phase): its slot (-1: none) and the parity of its phase.
+struct TcLastCommit {
+    int slot;
+    uint32_t parity;
+};
+__host__ __device__ constexpr TcLastCommit tc_last_commit(int count, int ring) {
+    return count > 0 ? TcLastCommit{(count - 1) % ring, (uint32_t)(((count - 1) / ring) & 1)} : TcLastCommit{-1, 0u};
+}
+static_assert(tc_last_commit(0, 4).slot == -1 && tc_last_commit(1, 4).slot == 0 && tc_last_commit(1, 4).parity == 0 &&
+                  tc_last_commit(4, 4).slot == 3 && tc_last_commit(4, 4).parity == 0 &&
+                  tc_last_commit(5, 4).slot == 0 && tc_last_commit(5, 4).parity == 1 &&
+                  tc_last_commit(9, 3).slot == 2 && tc_last_commit(9, 3).parity == 0,
+              "slot and phase of the last commit");
+
 // D (tensor memory) (+)= A B^T issued by the elected lane of a converged warp:
 // both operands in shared memory, or A in tensor memory (row i in lane i, two
 // bf16 K-values per 32-bit column)

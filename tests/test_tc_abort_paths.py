@@ -28,3 +28,15 @@ def test_no_lane_branches_on_its_own_wait(name):
     assert "tc_mbar_warp_wait" in code
     assert not re.findall(r"tc_mbar_(?:sleep|wait)_or_abort", code)
     assert not re.findall(r"if \(!?__all_sync", code), "a vote has to be kept: what follows must not use a lane's own value"
+
+
+def test_teardown_waits_for_the_last_unit_committed():
+    """Units of a tile given up half-way are in flight too: the count that the teardown
+    takes its slot and phase from goes up with every commit to a unit's mbarrier."""
+    code = _code("kron_tc.cu")
+    commits = re.findall(r"umma_commit\(&bar_full\[sl\]\);\s*(\S+)", code)
+    assert commits == ["++s_units;"]
+    assert code.count("++s_units") == 1 and "tc_mbar_wait(&bar_half" not in code
+    teardown = code[code.index("if (s_abort && tid == 0)"):code.index("tmem_dealloc")]
+    assert re.search(r"tc_last_commit\(s_units, S::kUnits\);\s*"
+                     r"if \(lc\.slot >= 0\) tc_mbar_wait\(&bar_full\[lc\.slot\], lc\.parity\);", teardown)
