@@ -304,10 +304,9 @@ __global__ void __launch_bounds__(288, 1) k_gram_async(const BlkDesc* __restrict
         const uint32_t el = tc_elect(), t0 = tc_uniform(tmem), tile0 = tc_uniform(tc_smem_addr(tiles));
         for (int st = 0; st < nst && ok; ++st) {
             const int b = st & 1;
-            ok = tc_mbar_sleep_or_abort(&conv_full[b], (uint32_t)((st >> 1) & 1), &s_abort);
+            ok = tc_mbar_warp_wait(&conv_full[b], (uint32_t)((st >> 1) & 1), &s_abort);
             // per-stage accumulator b was read back (stage st - 2)
-            if (ok && st >= 2) ok = tc_mbar_sleep_or_abort(&hi_free[b], (uint32_t)(((st - 2) >> 1) & 1), &s_abort);
-            ok = __all_sync(0xffffffffu, ok);
+            if (ok && st >= 2) ok = tc_mbar_warp_wait(&hi_free[b], (uint32_t)(((st - 2) >> 1) & 1), &s_abort);
             if (!ok) break;
             tc_fence_after();
             const uint64_t d0 = umma_desc_sw128(tile0 + (uint32_t)(b * 3 * kGTile));
@@ -343,8 +342,7 @@ __global__ void __launch_bounds__(288, 1) k_gram_async(const BlkDesc* __restrict
         for (int j = 0; j < NN; ++j) acc[j] = 0.f;
         auto read_back = [&](int st) {   // stage st's per-stage sums into acc, then release them
             const int b = st & 1;
-            bool r = tc_mbar_sleep_or_abort(&mma_done[b], (uint32_t)((st >> 1) & 1), &s_abort);
-            r = __all_sync(0xffffffffu, r);
+            const bool r = tc_mbar_warp_wait(&mma_done[b], (uint32_t)((st >> 1) & 1), &s_abort);
             tc_fence_after();
             if (r && reader) {
 #pragma unroll
@@ -364,10 +362,10 @@ __global__ void __launch_bounds__(288, 1) k_gram_async(const BlkDesc* __restrict
             gram_cp_commit();
             gram_cp_wait<1>();       // this thread's copies of stage st have landed
             tc_named_sync(1, 256);   // everyone's
-            if (s_abort) continue;
+            if (tc_warp_any(s_abort)) continue;
             // tile b was last read by the MMAs of stage st - 2
-            bool w = st < 2 || tc_mbar_sleep_or_abort(&mma_done[b], (uint32_t)(((st - 2) >> 1) & 1), &s_abort);
-            if (!__all_sync(0xffffffffu, w)) { s_abort = 1; continue; }
+            const bool w = st < 2 || tc_mbar_warp_wait(&mma_done[b], (uint32_t)(((st - 2) >> 1) & 1), &s_abort);
+            if (!w) { s_abort = 1; continue; }
             tc_fence_after();
             unsigned char* tile = tiles + b * 3 * kGTile;
             const double* rows = ring + (size_t)(st % kGRing) * kRows * kGK;
@@ -387,7 +385,7 @@ __global__ void __launch_bounds__(288, 1) k_gram_async(const BlkDesc* __restrict
             if (rwarp && st >= 1 && !read_back(st - 1)) s_abort = 1;
         }
         gram_cp_wait<0>();
-        ok = !s_abort;
+        ok = !tc_warp_any(s_abort);
         if (ok && rwarp) {
             ok = read_back(nst - 1);   // the last stage: its commit covers every MMA of the CTA
             if (ok && reader) {

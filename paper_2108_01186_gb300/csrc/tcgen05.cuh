@@ -252,6 +252,9 @@ __device__ __forceinline__ bool tc_mbar_warp_wait(uint64_t* bar, uint32_t parity
     return __all_sync(0xffffffffu, tc_mbar_sleep_or_abort(bar, parity, abort));
 }
 
+// The vote of a converged warp on a flag that another warp may set at any time
+__device__ __forceinline__ bool tc_warp_any(int flag) { return __any_sync(0xffffffffu, flag) != 0; }
+
 // named barrier over `count` threads (a multiple of 32) of the CTA
 __device__ __forceinline__ void tc_named_sync(int id, int count) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");

@@ -22,11 +22,12 @@ def test_the_voting_wait_returns_the_vote():
     assert re.search(r"return __all_sync\(0xffffffffu, tc_mbar_sleep_or_abort\(bar, parity, abort\)\);", body)
 
 
-@pytest.mark.parametrize("name", ["kron_tc.cu"])
+@pytest.mark.parametrize("name", ["kron_tc.cu", "gram_tc.cu"])
 def test_no_lane_branches_on_its_own_wait(name):
     code = _code(name)
     assert "tc_mbar_warp_wait" in code
     assert not re.findall(r"tc_mbar_(?:sleep|wait)_or_abort", code)
+    assert not re.findall(r"if \(!?s_abort\)|= !?s_abort;", code), "warps decide on the flag by a vote"
     assert not re.findall(r"if \(!?__all_sync", code), "a vote has to be kept: what follows must not use a lane's own value"
 
 
