@@ -124,12 +124,13 @@ __global__ void __launch_bounds__(256, 2) k_hamiltonian_ix(const BlkDesc* __rest
     __syncthreads();
     {   // the largest exponent among this tile and those its taps reach (periodic: the orbital's)
         const int ntx = (nx + kTileX - 1) / kTileX, nty = (ny + kTileY - 1) / kTileY;
-        int e = 0;
+        int e = 0, bad = 0;   // (apart: a flag in e would outweigh every later exponent)
+        auto take = [&](int v) {
+            e = max(e, v & (kExpBad - 1));
+            bad |= v & kExpBad;
+        };
         if (per) {
-            for (int t = tid; t < D.ntile; t += 256) {
-                const int v = texp[P.first + t];
-                e = max(e, v & (kExpBad - 1)) | ((e | v) & kExpBad);
-            }
+            for (int t = tid; t < D.ntile; t += 256) take(texp[P.first + t]);
         } else if (tid < 32) {
             const int kx = P.x0 / kTileX, ky = P.y0 / kTileY;
             const int kz0 = max(P.z0 - kHalf, 0) / D.tz, kz1 = min(P.z1 + kHalf - 1, nz - 1) / D.tz;
@@ -141,12 +142,10 @@ __global__ void __launch_bounds__(256, 2) k_hamiltonian_ix(const BlkDesc* __rest
                 else jy += 2 * tid - 5;
                 ok = jx >= 0 && jx < ntx && jy >= 0 && jy < nty;
             }
-            if (ok) e = texp[P.first + ((long long)jz * nty + jy) * ntx + jx];
+            if (ok) take(texp[P.first + ((long long)jz * nty + jy) * ntx + jx]);
         }
-        if (e) {
-            atomicMax(&s_exp, e & (kExpBad - 1));
-            if (e & kExpBad) s_bad = 1;
-        }
+        if (e) atomicMax(&s_exp, e);
+        if (bad) s_bad = 1;
         __syncthreads();
     }
     const int et = s_exp;             // |psi| < 2^(et - 1022)
