@@ -467,8 +467,7 @@ int flosic_create(flosic_ctx** out, const flosic_system* sys, int nsys, const fl
             for (int b = 0; b < c->nblk; ++b) { nl[b] = 1; coarsest[b] = 0; }
         }
         const size_t tsz = (o.precision == FLOSIC_FP64) ? sizeof(double) : sizeof(float);
-        // the levels that k_mg_coarse takes: from the first one of at most mg_fuse_max
-        // points that fits in shared memory with those below it (always the coarsest)
+        // the levels that k_mg_coarse takes (mg_fuse), as far as they fit in shared memory
         std::vector<int> fused = coarsest;
         for (int b = 0; b < c->nblk && M.enabled; ++b) {
             const BlkDesc& B = c->blk[b];
@@ -477,7 +476,8 @@ int flosic_create(flosic_ctx** out, const flosic_system* sys, int nsys, const fl
             };
             while (fused[b] > 0) {
                 const int l = fused[b] - 1;
-                if ((long long)(B.nx >> l) * (B.ny >> l) * (B.nz >> l) > mg_fuse_max(tsz) || bytes(l) > kMgSmemMax) break;
+                const long long G = (long long)(B.nx >> l) * (B.ny >> l) * (B.nz >> l);
+                if (bytes(l) > kMgSmemMax || !mg_fuse(tsz, l, G, c->norb, c->num_sms)) break;
                 fused[b] = l;
             }
             M.fused_max = std::max(M.fused_max, fused[b]);

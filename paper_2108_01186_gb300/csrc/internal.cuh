@@ -79,12 +79,26 @@ inline int tile_depth(int max_tz, int min_tz, int num_sms, Tiles tiles) {
 }
 constexpr int kCoarseSweeps = 40;      // damped-Jacobi sweeps on the coarsest level
 constexpr int kCoarseMax = 2000;       // largest coarsest level (points) kept in shared memory
-// Levels that the V-cycle runs in one launch, a CTA per orbital (k_mg_coarse):
-// in float32 as many as fit in shared memory (24^3 points and those below); in
-// float64 levels of up to 2000 points, where a CTA's float64 pipe (1.7 FMA per
-// cycle) takes less than the 30 us of the level's four launches.
+// Levels that the V-cycle runs in one launch, a CTA per orbital in shared memory
+// (k_mg_coarse): the coarsest one always, and from there up every level of G
+// points that fits and takes less time there than in its own four launches.
+//  * There, the orbitals run in waves of one CTA per SM, 2.5 ns per point and
+//    wave in float32 (24^3 points 35 us, 16^3 10 us).
+//  * The four launches take 20 us and 9.5 ps per point and orbital on level 0,
+//    20 ps below it (shallow tiles, weighted diagonals).
+// V-cycle and rest of an iteration, level fused / not: 24^3 points as level 0 88 / 74
+// us at 10 orbitals, 125 / 130 at 150, 184 / 157 at 160, 873 / 738 at 1300; as level 1
+// of 48^3 137 / 124 at 10, 501 / 525 at 150, 572 / 566 at 160, 889 / 917 at 300; 16^3 as
+// level 0 59 / 70 at 10, 110 / 120 at 300, 406 / 368 at 1300.
+// float64: levels of up to 2000 points, where a CTA's float64 pipe (1.7 FMA per
+// cycle) takes less than the launches for any number of orbitals (12^3 points of
+// 24^3: 144 / 151 us at 10, 5078 / 5478 at 1300).
 constexpr size_t kMgSmemMax = 200 * 1024;
-constexpr long long mg_fuse_max(size_t elem) { return elem == sizeof(float) ? 14000 : 2000; }
+inline bool mg_fuse(size_t elem, int level, long long G, int norb, int num_sms) {
+    if (elem != sizeof(float)) return G <= 2000;
+    const double waves = (double)((norb + num_sms - 1) / num_sms);
+    return waves * 2.5e-3 * (double)G < 20.0 + (level == 0 ? 9.5e-6 : 20e-6) * (double)norb * (double)G;   // us
+}
 long long mg_coarse_elems(int nx, int ny, int nz, int nlev);
 // planes of a tile staged with the 6-point x/y halo by the z-marching sweeps
 constexpr int kPX = kTileX + 2 * kHalf;   // staged plane width
