@@ -524,7 +524,7 @@ int flosic_create(flosic_ctx** out, const flosic_system* sys, int nsys, const fl
                             if (m & (1 << k)) dd += (double)D.cl[k] - 2.0;
                         D.idd[m] = (float)(1.0 / dd);
                     }
-                    D.tz = depth;
+                    D.tz = tile_split(D.nz, depth);
                     D.per = (l == 0) ? B.per : 0;
                     const int tx = (D.nx + kTileX - 1) / kTileX, ty = (D.ny + kTileY - 1) / kTileY,
                               tz = (D.nz + D.tz - 1) / D.tz;

@@ -77,6 +77,13 @@ inline int tile_depth(int max_tz, int min_tz, int num_sms, Tiles tiles) {
     while (tz > min_tz && tiles(tz) < 3LL * num_sms) tz /= 2;
     return tz;
 }
+// A block's tile depth: its planes in as many tiles, of equal depth (24 planes at
+// depth 16 as 16 + 8 left half the SMs with twice the others' work: float64 solves of
+// 24^3 x 150 16.0 ms, as 12 + 12 13.0 ms).
+inline int tile_split(int nz, int depth) {
+    const int n = (nz + depth - 1) / depth;
+    return (nz + n - 1) / n;
+}
 constexpr int kCoarseSweeps = 40;      // damped-Jacobi sweeps on the coarsest level
 constexpr int kCoarseMax = 2000;       // largest coarsest level (points) kept in shared memory
 // Levels that the V-cycle runs in one launch, a CTA per orbital in shared memory
