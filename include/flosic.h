@@ -27,6 +27,8 @@
  *    per-orbital scalars (U, Exc, iters, conv_flags) are packed per block;
  *    V_avg is one [G] array per block; E_sic and gE hold one value per
  *    system.  flosic_layout() returns every packed size.
+ *  - Device arrays need the alignment of their elements only; the wide accesses
+ *    of arrays on 16-byte boundaries give way to single ones otherwise.
  *  - Every call is asynchronous on `stream` (a cudaStream_t, passed as
  *    void*), except that calls whose result can fail on the device
  *    (flosic_build_flos: ILLCOND/NONFINITE, flosic_orbital_poisson: NOCONV)
@@ -174,7 +176,7 @@ int flosic_layout(const flosic_ctx* ctx, int64_t* out);
  * transforms run on the tensor cores (KRON solver; the autotuner's pick
  * when autotune is 1), bit 1 = its refinement update is staged by the copy
  * engine, bit 2 = its overlap Gram stages psi with asynchronous copies
- * (MIXED).  Errors: ARG. */
+ * (MIXED, psi on a 16-byte boundary).  Errors: ARG. */
 int flosic_block_paths(const flosic_ctx* ctx, int* out);
 
 /* Steps a1-a5 (Sec. II.B, Eqs. 6-8, Loewdin of Sec. I.B):

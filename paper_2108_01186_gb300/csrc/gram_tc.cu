@@ -78,7 +78,7 @@ __host__ __device__ constexpr int gram_pack() { return (32 * NB <= 64) ? 128 / (
 template <int NB>   // NB = orbital rows per sub-chunk / 32 (1 .. 4)
 __global__ void __launch_bounds__(256, NB <= 2 ? 2 : 1) k_gram_tc(const BlkDesc* __restrict__ blk, const double* __restrict__ psi,
                                                     float* __restrict__ part, const long long* __restrict__ part_off,
-                                                    int* __restrict__ status) {
+                                                    int all, int* __restrict__ status) {
     extern __shared__ unsigned char g_smem_raw[];
     __shared__ uint64_t mbar[kGStages];
     __shared__ uint32_t tmem_base;
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(256, NB <= 2 ? 2 : 1) k_gram_tc(const BlkDesc*
     constexpr int kSub = kGChunk / P;                // points per sub-chunk
     constexpr uint32_t kCols = (2 * MN <= 128) ? 128 : 256;
     const BlkDesc& B = blk[blockIdx.y];
-    if (B.gtma) return;                              // k_gram_tma's block
+    if (B.gtma && !all) return;                      // k_gram_async's block
     const int N = B.N;
     const long long g_begin = (long long)blockIdx.x * kGChunk;
     if (g_begin >= B.G) return;                      // whole CTA
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(256, NB <= 2 ? 2 : 1) k_gram_tc(const BlkDesc*
 
 // The same sums with the float64 psi tiles brought to shared memory by
 // asynchronous copies (cp.async, 16 bytes each; blocks whose G and offset are
-// even, so every piece is 16-byte aligned): a ring of kGRing stages, the copies
+// even, of a psi on a 16-byte boundary, so every piece is aligned): a ring of kGRing stages, the copies
 // of stage st + 1 in flight while stage st is converted and multiplied, rows
 // past N and points past G zero-filled by the copy.  The warps convert rows
 // from shared memory (lane l: points 2l, 2l + 1 of one row) into the same
@@ -474,7 +474,8 @@ cudaError_t setup_gram_tc() {
     return e;
 }
 
-// blocks whose psi rows the asynchronous-copy kernel can take (16-byte pieces)
+// blocks whose psi rows the asynchronous-copy kernel can take (16-byte pieces of a
+// psi that starts on a 16-byte boundary itself)
 bool gram_async_eligible(const BlkDesc& B) { return B.G % 2 == 0 && B.off % 2 == 0; }
 
 void launch_gram_tc(const flosic_ctx* c, const double* psi, cudaStream_t s) {
@@ -499,7 +500,9 @@ void launch_gram_tc(const flosic_ctx* c, const double* psi, cudaStream_t s) {
         for (const auto& b : c->blk) cm->ov_flops += 2.0 * b.N * b.N * (double)b.G;
     }
     int n_async = 0;
-    for (const auto& b : c->blk) n_async += b.gtma;
+    if (aligned16(psi))
+        for (const auto& b : c->blk) n_async += b.gtma;
+    const int all = n_async == 0;   // k_gram_tc takes every block
     if (n_async > 0) {   // blocks with 16-byte aligned rows: copies staged asynchronously
         if (nb <= 1) k_gram_async<1><<<grid, 288, kGAsyncSmem, s>>>(c->d_blk, psi, part, off, c->ws.status);
         else if (nb == 2) k_gram_async<2><<<grid, 288, kGAsyncSmem, s>>>(c->d_blk, psi, part, off, c->ws.status);
@@ -508,10 +511,10 @@ void launch_gram_tc(const flosic_ctx* c, const double* psi, cudaStream_t s) {
         note_launch(cm);
     }
     if (n_async < c->nblk) {   // the others: thread loads
-        if (nb <= 1) k_gram_tc<1><<<grid, 256, kGSmem, s>>>(c->d_blk, psi, part, off, c->ws.status);
-        else if (nb == 2) k_gram_tc<2><<<grid, 256, kGSmem, s>>>(c->d_blk, psi, part, off, c->ws.status);
-        else if (nb == 3) k_gram_tc<3><<<grid, 256, kGSmem, s>>>(c->d_blk, psi, part, off, c->ws.status);
-        else k_gram_tc<4><<<grid, 256, kGSmem, s>>>(c->d_blk, psi, part, off, c->ws.status);
+        if (nb <= 1) k_gram_tc<1><<<grid, 256, kGSmem, s>>>(c->d_blk, psi, part, off, all, c->ws.status);
+        else if (nb == 2) k_gram_tc<2><<<grid, 256, kGSmem, s>>>(c->d_blk, psi, part, off, all, c->ws.status);
+        else if (nb == 3) k_gram_tc<3><<<grid, 256, kGSmem, s>>>(c->d_blk, psi, part, off, all, c->ws.status);
+        else k_gram_tc<4><<<grid, 256, kGSmem, s>>>(c->d_blk, psi, part, off, all, c->ws.status);
         note_launch(cm);
     }
     if (timed) {

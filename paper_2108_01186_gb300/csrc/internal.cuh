@@ -680,11 +680,16 @@ template <class T> struct Vec;
 template <> struct Vec<float> { using type = float4; static constexpr int n = 4; };
 template <> struct Vec<double> { using type = double2; static constexpr int n = 2; };
 
+// Is a caller's array aligned for 16-byte accesses?  (The workspace's arrays are;
+// a caller's need only be aligned to their elements.)
+__host__ __device__ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 // Elementwise sweep over one tile, vectorised along x when the rows are
-// aligned (nx a multiple of the vector width); body(g, n) handles n
-// consecutive points starting at flat index g (n = vector width, or 1).
+// aligned (nx a multiple of the vector width, and `aligned`: every array that
+// body accesses by vectors is); body(g, n) handles n consecutive points
+// starting at flat index g (n = vector width, or 1).
 template <class T, class Body>
-__device__ __forceinline__ void tile_elementwise(const LvlDesc& D, const TilePos& P, Body body) {
+__device__ __forceinline__ void tile_elementwise(const LvlDesc& D, const TilePos& P, Body body, bool aligned = true) {
     constexpr int V = Vec<T>::n;
     constexpr int XG = kTileX / V;               // vector groups per row
     constexpr int RPI = 256 / XG;                // rows per pass
@@ -692,7 +697,7 @@ __device__ __forceinline__ void tile_elementwise(const LvlDesc& D, const TilePos
     const int xg = tid % XG, r0 = tid / XG;
     const int nz = P.z1 - P.z0;
     const int nrows = kTileY * nz;
-    const bool vec = (D.nx % V == 0) && (P.base % V == 0);
+    const bool vec = (D.nx % V == 0) && (P.base % V == 0) && aligned;
     const int x = P.x0 + xg * V;
 #pragma unroll 4
     for (int row = r0; row < nrows; row += RPI) {
@@ -711,7 +716,7 @@ __device__ __forceinline__ void tile_elementwise(const LvlDesc& D, const TilePos
 
 // Same sweep, passing the coordinates of the first point: body(x, y, z, g, n).
 template <class T, class Body>
-__device__ __forceinline__ void tile_rows(const LvlDesc& D, const TilePos& P, Body body) {
+__device__ __forceinline__ void tile_rows(const LvlDesc& D, const TilePos& P, Body body, bool aligned = true) {
     constexpr int V = Vec<T>::n;
     constexpr int XG = kTileX / V;
     constexpr int RPI = 256 / XG;
@@ -719,7 +724,7 @@ __device__ __forceinline__ void tile_rows(const LvlDesc& D, const TilePos& P, Bo
     const int xg = tid % XG, r0 = tid / XG;
     const int nz = P.z1 - P.z0;
     const int nrows = kTileY * nz;
-    const bool vec = (D.nx % V == 0) && (P.base % V == 0);
+    const bool vec = (D.nx % V == 0) && (P.base % V == 0) && aligned;
     const int x = P.x0 + xg * V;
 #pragma unroll 2
     for (int row = r0; row < nrows; row += RPI) {

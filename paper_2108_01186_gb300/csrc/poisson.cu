@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(256) k_pcg_update_t(const BlkDesc* __restrict_
             r[g] = rv;
             rr += rv * rv;
         }
-    });
+    }, aligned16(x));   // (in float64 x is the caller's V)
     if (tile_arrive(rr, st.part, blockIdx.x, st.count + P.o, D.ntile, scratch)) {
         const double sum = tile_gather(st.part, P.first, D.ntile, scratch);
         if (linear_tid() == 0) {

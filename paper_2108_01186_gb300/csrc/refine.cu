@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(256) k_ff_init(const BlkDesc* __restrict__ blk
                 if (p32) p32[q + k] = bh;
             }
         }
-    });
+    }, !warm || aligned16(V));
     if (tile_arrive(bb, st.part, blockIdx.x, st.count + P.o, D.ntile, scratch)) {
         const double sum = tile_gather(st.part, P.first, D.ntile, scratch);
         if (linear_tid() == 0) {
@@ -729,7 +729,7 @@ __global__ void __launch_bounds__(256) k_join_ff(const BlkDesc* __restrict__ blk
             return;
         }
         for (int k = 0; k < n; ++k) V[g + k] = ff2d(x[g + k]);
-    });
+    }, aligned16(V));
 }
 
 static dim3 tile_threads() { return dim3(kTileX, kTileY / 2); }
