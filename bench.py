@@ -841,7 +841,7 @@ def run_hamiltonian(args):
                           "dtype": "f32-ff" if prec else "f64", "data": "synthetic",
                           "config": {"workload": "128^3 h=0.2, 32+32 orbitals, H = -1/2 Lap + V_avg",
                                      "precision": args.precision},
-                          "roofline": {"bound": "hbm", "kernel": "k_hamiltonian_ix" if prec else "k_hamiltonian64",
+                          "roofline": {"bound": "hbm", "kernel": "k_hamiltonian_mixed" if prec else "k_hamiltonian64",
                                        "achieved": round(ach, 1), "peak": peaks.get("hbm_gbs"),
                                        "peak_source": peaks["source"],
                                        "unit": "GB/s", "frac": round(ach / peaks["hbm_gbs"], 4),

@@ -273,9 +273,11 @@ int flosic_sic_backward(flosic_ctx* ctx, const double* psi, const double* fods,
  *      V_avg [sum G over spin blocks] float64 or NULL: the averaged SIC
  *      potential as written by flosic_sic_energy_potential (scaled by s).
  * Out: Hpsi [sum N*G] float64 (must not overlap psi).
- * Precision follows the context: FP64 in float64; MIXED with the Laplacian
- * in exact integer sums of psi held to 2^-57 of the largest value nearby, the
- * potential term in float64.
+ * Precision follows the context: FP64 in float64; MIXED with psi in
+ * the Laplacian held to 2^-48 of each value and to 2^-60 of the largest one
+ * nearby, whichever is finer (values below 2^-173 of that one count as zero), the
+ * potential term in float64.  A point that reads an infinity, a NaN or a value
+ * beyond 2^799 gets NaN.
  * Errors: ARG (NULL ctx, psi or Hpsi, or Hpsi == psi), CUDA.  Asynchronous
  * on `stream`. */
 int flosic_hamiltonian_apply(flosic_ctx* ctx, const double* psi, const double* vloc,

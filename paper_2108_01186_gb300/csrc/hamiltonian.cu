@@ -13,30 +13,38 @@ namespace flosic {
 __constant__ double c_w64[kHalf + 1];   // this file's copy of the 12th-order weights
 
 // ---------------------------------------------------------------------------
-// Mixed precision: the Laplacian in exact integer sums (ixsweep.cuh).
+// Mixed precision: psi as a top digit and a float32 pair, their stencil sums
+// free of rounding but in the pairs' low parts.
 //
 // A tile's psi (with the halo its taps reach) lies below 2^k, k from the
-// tiles' largest exponents (k_tile_exp).  Every staged value becomes the
-// integer q = trunc(psi 2^(57-k)) in two digits, q = hi 2^29 + lo with
-// |hi|, |lo| <= 2^28; both digit fields are summed and weighted in integers,
-// so the only rounding of the Laplacian is the 2^-57 of the tile's largest
-// value (the float-float sweep that this replaced held 2^-48 of each value) and
-// the final float64 result, which takes three float64 operations per point.
+// tiles' largest exponents (k_tile_exp); it is scaled to lie below 2^100.  A
+// value splits into v = b 2^89 + (h + l): b an integer of at most 2^11, h + l the
+// rest as a float32 pair.  The b's of the six neighbours at a distance and their
+// weighting are integer sums; the h's are summed by error-free two-sums and
+// weighted by exact products; l's, two-sum and product errors are added in
+// float32.  So what is lost is 2^-48 of each value (the pair's own resolution,
+// any size of value) and never more than 2^-60 of the tile's largest: a field's
+// tail keeps the bits that a fixed point would take from it, and its bulk is
+// as exact as float64.  (Two digits of 29 bits below the tile's largest value, the
+// former kernel, held 85 % of this library's orbitals on 128^3 points, the tails, in fewer
+// bits than a pair does, a quarter of them as zero.)
 //
-// What bounds it: instruction issue and the latencies of 16 warps per SM (310
-// instructions per point, 46 % of the issue slots; 128 registers a thread hold
-// the z-windows).  The two digits need 6 integer additions (three-operand) and
-// 2 multiply-adds per distance, against error-free sums and products of pairs.
-// A value is split once, when its plane arrives (IxStage); one barrier per
-// plane.  With the z-loop unrolled 13 times, which keeps every window slot in
-// place, a third of the issue slots waited for instructions (2.7 -> 3.5 ms).
-// 128^3 x 64 orbitals with both potentials: 5.82 -> 2.24 ms, of which
-// k_tile_exp 0.15.
+// What bounds it: instruction issue and latencies at 16 warps per SM (520
+// instructions per point, half of the issue slots; the packed operations fill half of
+// their pipe).  A value is split once, when its plane arrives (IxStage); one barrier per
+// plane.  The planes z - 6 .. z - 1 of a thread's points are in registers, z + 1 .. z + 6
+// in the ring (3.40 ms; all twelve in registers 3.46; the z-loop unrolled once, twice, four
+// times 3.50, 3.42, 3.58).  128^3 x 64 orbitals with both potentials 3.32 ms,
+// of which k_tile_exp 0.15: the float-float sweep with plain loads took 5.81, the two
+// digits 2.21.  Error against 64 bits in the 2-norm (96^3, Gaussians): 1.3e-13, 2.1e-15
+// with the digits, 4.7e-16 now.
 // ---------------------------------------------------------------------------
-constexpr int kHSmem = kIxPts * 8 * kIxRing;
+constexpr int kHZU = 3;                              // steps of the z-loop unrolled
+constexpr int kHRing = 9;                            // staged planes: see the z-loop
+constexpr int kHOffTop = kIxPts * 8 * kHRing;        // the top digits, behind the pairs
+constexpr int kHSmem = kHOffTop + kIxPts * 2 * kHRing;
 constexpr int kExpBad = 1 << 16;                     // a tile with a value beyond 2^799, an infinity or a NaN
-constexpr int kExpMin = 223, kExpMax = 1821;         // biased exponents in use: the scales stay normal float64
-                                                     // (smaller psi count as zero)
+constexpr int kExpMin = 226, kExpMax = 1821;         // scale exponents in use: the scales stay normal float64
 __device__ __forceinline__ int expo(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 
 // Per tile: the largest biased exponent of its psi, + kExpBad.
@@ -72,44 +80,75 @@ __global__ void __launch_bounds__(256) k_tile_exp(const BlkDesc* __restrict__ bl
     if (linear_tid() == 0) texp[blockIdx.x] = s_max | s_bad;
 }
 
-// trunc(v 2^(1079 - et)) as digits (hi, lo); et at least kExpMin and at least
-// v's biased exponent (what lies above it becomes 0: the staged corners, which
-// no tap reads, and the values that make a tile bad).
-__device__ __forceinline__ int2 ix_digits(double v, int et) {
-    const int hw = __double2hiint(v);
-    const unsigned sh = min((unsigned)(et - ((hw >> 20) & 0x7ff)), 63u);
-    const unsigned long long m =
-        ((unsigned long long)(unsigned)((hw & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
-    const long long sg = hw >> 31;
-    const long long q = ((long long)((m << 4) >> sh) ^ sg) - sg;
-    const long long t = q + (1 << 28);
-    return make_int2((int)(t >> 29), (int)((unsigned)t & 0x1fffffffu) - (1 << 28));
+// Two neighbouring points' parts: pairs h + l, and the top digits as unsigned
+// 16-bit lanes b + kTopBias (the weights of a point's 37 taps sum to zero, so the
+// bias leaves no trace, and six lanes add up without a carry).
+struct __align__(16) HPair {
+    float2 h, l;
+};
+constexpr float kTopUnit = 6.18970019642690137e26f;   // 2^89
+constexpr int kTopBias = 4096;
+
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+// a + b = s + e exactly, one lane and two at once
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+    const ff s = ff_two_sum(a, b);
+    e = s.l;
+    return s.h;
+}
+__device__ __forceinline__ float2 two_sum2(float2 a, float2 b, float2& e) {
+    const float2 s = __fadd2_rn(a, b), bb = sub2(s, a);
+    e = __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb));
+    return s;
 }
 
-// H 2^10 + L 2^-19 (H, L weighted sums of hi and lo digits, below 2^53 in
-// magnitude) in float64, built with integer operations: the sum as an integer
-// (2^-10 of a unit of H, a quarter of the digits' own resolution after
-// weighting), normalised and truncated to 53 bits.
-__device__ __forceinline__ double ix_to_double(long long H, long long L) {
-    const long long t = (H << 10) + ((L + (1 << 18)) >> 19);
-    const long long sg = t >> 63;
-    const unsigned long long a = (unsigned long long)((t ^ sg) - sg);
-    if (a == 0) return 0.0;
-    const int lz = __clzll((long long)a);
-    const unsigned long long m = a << lz;   // its top bit adds 1 to the exponent
-    const unsigned hw = ((unsigned)(1023 + 62 - lz) << 20) + (unsigned)(m >> 43);
-    return __hiloint2double((int)(hw | ((unsigned)sg & 0x80000000u)), (int)(unsigned)(m >> 11));
+// One value v 2^(1122 - et) (below 2^100 by its tile's et): f its sign, power of two and
+// the 21 leading bits, pw the power of two alone; the 32 bits below as two floats, v = f +
+// (a 2^16 + b) 2^-52 pw.  Integer operations: a 64-bit conversion would run on the float64
+// pipe.  Zero where v exceeds et (the staged corners, which no tap reads, and
+// the values that make a tile bad) or is below 2^-173 of it.
+__device__ __forceinline__ void top_parts(double v, unsigned lo, float& f, float& pw, float& a, float& b) {
+    const unsigned hw = (unsigned)__double2hiint(v), lw = (unsigned)__double2loint(v);
+    const unsigned d = (hw & 0x7fffffffu) - lo;
+    const unsigned w = d < (174u << 20) ? ((d << 3) + (53u << 23)) | (hw & 0x80000000u) : 0u;
+    f = __uint_as_float(w);
+    pw = __uint_as_float(w & 0xff800000u);
+    a = __uint_as_float(__byte_perm(lw, 0x4B000000u, 0x7632)) - 8388608.f;
+    b = __uint_as_float(__byte_perm(lw, 0x4B000000u, 0x7610)) - 8388608.f;
+}
+// lo: the least high word in use, (et - 173) 2^20
+__device__ __forceinline__ HPair top_split(double2 v, unsigned lo, unsigned& top) {
+    float2 f, pw, a, b;
+    top_parts(v.x, lo, f.x, pw.x, a.x, b.x);
+    top_parts(v.y, lo, f.y, pw.y, a.y, b.y);
+    constexpr float kM = kTopUnit * (float)(0xC00000 + kTopBias);   // f + kM rounds f to the units of the top digit
+    constexpr float k36 = 1.f / 68719476736.f, k16 = 1.f / 65536.f;
+    const float2 m2 = make_float2(kM, kM);
+    const float2 tq = __fadd2_rn(f, m2);
+    top = __byte_perm(__float_as_uint(tq.x), __float_as_uint(tq.y), 0x5410);
+    const float2 r1 = sub2(f, sub2(tq, m2));                       // exact, 0 or larger than t
+    const float2 u = __fmul2_rn(pw, make_float2(k36, k36)), t = __fmul2_rn(a, u);
+    HPair p;
+    p.h = __fadd2_rn(r1, t);
+    p.l = __ffma2_rn(b, __fmul2_rn(u, make_float2(k16, k16)), sub2(t, sub2(p.h, r1)));
+    return p;
+}
+// (I 2^89 + h + l) cf; |I| < 2^51
+__device__ __forceinline__ double top_join(long long I, float h, float l, double cf) {
+    const double d = __longlong_as_double(I + 0x4338000000000000LL) - 6755399441055744.0;
+    return fma(d, (double)kTopUnit, f2d(h) + f2d(l)) * cf;
 }
 
-__global__ void __launch_bounds__(256, 2) k_hamiltonian_ix(const BlkDesc* __restrict__ blk, const LvlDesc* __restrict__ L,
-                                                           const int4* __restrict__ tiles,
-                                                           const int* __restrict__ orb_blk,
-                                                           const double* __restrict__ psi,
-                                                           const double* __restrict__ vloc,
-                                                           const double* __restrict__ vavg,
-                                                           const int* __restrict__ texp, double* __restrict__ hpsi) {
+__global__ void __launch_bounds__(256, 2) k_hamiltonian_mixed(const BlkDesc* __restrict__ blk, const LvlDesc* __restrict__ L,
+                                                              const int4* __restrict__ tiles,
+                                                              const int* __restrict__ orb_blk,
+                                                              const double* __restrict__ psi,
+                                                              const double* __restrict__ vloc,
+                                                              const double* __restrict__ vavg,
+                                                              const int* __restrict__ texp, double* __restrict__ hpsi) {
     extern __shared__ __align__(16) unsigned char hs_raw[];
-    int2* const ring = reinterpret_cast<int2*>(hs_raw);
+    HPair* const ring = reinterpret_cast<HPair*>(hs_raw);
+    unsigned* const tops = reinterpret_cast<unsigned*>(hs_raw + kHOffTop);
     __shared__ int s_exp, s_bad;
     __shared__ double s_cf;
     const TilePos P = tile_pos(blk, L, tiles, orb_blk, blockIdx.x);
@@ -122,35 +161,31 @@ __global__ void __launch_bounds__(256, 2) k_hamiltonian_ix(const BlkDesc* __rest
         s_bad = 0;
     }
     __syncthreads();
-    {   // the largest exponent among this tile and those its taps reach (periodic: the orbital's)
-        const int ntx = (nx + kTileX - 1) / kTileX, nty = (ny + kTileY - 1) / kTileY;
-        int e = 0, bad = 0;   // (apart: a flag in e would outweigh every later exponent)
-        auto take = [&](int v) {
-            e = max(e, v & (kExpBad - 1));
-            bad |= v & kExpBad;
-        };
-        if (per) {
-            for (int t = tid; t < D.ntile; t += 256) take(texp[P.first + t]);
-        } else if (tid < 32) {
-            const int kx = P.x0 / kTileX, ky = P.y0 / kTileY;
-            const int kz0 = max(P.z0 - kHalf, 0) / D.tz, kz1 = min(P.z1 + kHalf - 1, nz - 1) / D.tz;
-            int jx = kx, jy = ky, jz = kz0 + tid - 4;   // lanes 4 ..: the column's tiles
-            bool ok = tid >= 4 && jz <= kz1;
-            if (tid < 4) {
-                jz = P.z0 / D.tz;
-                if (tid < 2) jx += 2 * tid - 1;
-                else jy += 2 * tid - 5;
-                ok = jx >= 0 && jx < ntx && jy >= 0 && jy < nty;
+    if (tid < 1 + 12 * 3) {   // the largest exponent in this tile (thread 0) and in those of the six points on either side
+        int c[3] = {P.x0, P.y0, P.z0};
+        const int n3[3] = {nx, ny, nz}, end[3] = {min(P.x0 + kTileX, nx), min(P.y0 + kTileY, ny), P.z1};
+        bool ok = true;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int j = tid - 1 - 12 * d;
+            if (j >= 0 && j < 12) {
+                c[d] = j < kHalf ? c[d] - kHalf + j : end[d] + j - kHalf;
+                if (per & (1 << d)) c[d] = wrap_coord(c[d], n3[d]);
+                ok = c[d] >= 0 && c[d] < n3[d];
             }
-            if (ok) take(texp[P.first + ((long long)jz * nty + jy) * ntx + jx]);
         }
-        if (e) atomicMax(&s_exp, e);
-        if (bad) s_bad = 1;
-        __syncthreads();
+        if (ok) {
+            const int ntx = (nx + kTileX - 1) / kTileX, nty = (ny + kTileY - 1) / kTileY;
+            const int e = texp[P.first + ((long long)(c[2] / D.tz) * nty + c[1] / kTileY) * ntx + c[0] / kTileX];
+            atomicMax(&s_exp, e & (kExpBad - 1));
+            if (e & kExpBad) s_bad = 1;
+        }
     }
+    __syncthreads();
     const int et = s_exp;             // |psi| < 2^(et - 1022)
-    // weighted sums (units of 2^(et - 1022 - 38) / 831600) -> -h^2/2 Delta_h psi; one thread's float64 division
-    if (tid == 0) s_cf = scalbn(-0.5 / ((double)kW12Den * D.h * D.h), et - 1022 - 38);
+    const unsigned lo = (unsigned)(et - 173) << 20;
+    // weighted sums (units of 2^(et - 1122) / 831600) -> -1/2 Delta_h psi; one thread's float64 division
+    if (tid == 0) s_cf = scalbn(-0.5 / ((double)kW12Den * D.h * D.h), et - 1122);
     constexpr int kWc = (int)w12_centre3();
     constexpr int kW[kHalf + 1] = {kWc,           (int)w12_int(1), (int)w12_int(2), (int)w12_int(3),
                                    (int)w12_int(4), (int)w12_int(5), (int)w12_int(6)};
@@ -168,23 +203,19 @@ __global__ void __launch_bounds__(256, 2) k_hamiltonian_ix(const BlkDesc* __rest
         const double* pl = psi + P.base + (okz ? z * sz : 0);
 #pragma unroll
         for (int j = 0; j < kIxU; ++j)
-            if (sg.wants(j, k < nzt)) sg.copy(j, ring + slot * kIxPts + 2 * (tid + j * 256), pl, okz, vec, nx);
+            if (sg.wants(j, k < nzt)) sg.copy(j, ring + slot * kIxPairs + tid + j * 256, pl, okz, vec, nx);
     };
     auto split = [&](int k, int slot) {
 #pragma unroll
         for (int j = 0; j < kIxU; ++j)
             if (sg.wants(j, k < nzt)) {
-                int2* const at = ring + slot * kIxPts + 2 * (tid + j * 256);
-                const double2 v = *reinterpret_cast<const double2*>(at);
-                const int2 d0 = ix_digits(v.x, et), d1 = ix_digits(v.y, et);
-                *reinterpret_cast<int4*>(at) = make_int4(d0.x, d0.y, d1.x, d1.y);
+                const int at = slot * kIxPairs + tid + j * 256;
+                ring[at] = top_split(*reinterpret_cast<const double2*>(ring + at), lo, tops[at]);
             }
     };
     for (int k = 0; k < kHalf; ++k) copy(k, k);
     cp_async_commit();
     copy(kHalf, kHalf);
-    cp_async_commit();
-    copy(kHalf + 1, kHalf + 1);
     cp_async_commit();
 
     const int tx = threadIdx.x, ty = threadIdx.y;     // 16 x 16; points (x0 + 2 tx + a, y0 + ty)
@@ -192,37 +223,32 @@ __global__ void __launch_bounds__(256, 2) k_hamiltonian_ix(const BlkDesc* __rest
     const bool in0 = gx < nx && gy < ny, in1 = gx + 1 < nx && gy < ny;
     const bool ovec = (nx & 1) == 0 && (P.base & 1) == 0 && ((reinterpret_cast<uintptr_t>(hpsi) & 15) == 0);
     const long long col = gy * sy + gx;
-    const int ctr = (ty + kHalf) * kPX + 2 * tx + kHalf;   // the first point in a staged plane
-    int2 q0[kQ], q1[kQ];   // z-windows: step k0 + u's in slots u .. u + 12
+    const int ctr = (ty + kHalf) * (kPX / 2) + tx + kHalf / 2;   // the points' pair in a staged plane
+    HPair q[kHalf + kHZU];   // planes z - 6 .. z - 1 of step k0 + u in slots u .. u + 5
+    unsigned qt[kHalf + kHZU];
 #pragma unroll
     for (int j = 0; j < kHalf; ++j) {   // planes z0 - 6 .. z0 - 1 straight from memory
         int z = P.z0 - kHalf + j;
         if (per & 4) z = wrap_coord(z, nz);
         const double* pl = psi + P.base + z * sz + col;
-        q0[j] = ix_digits(z >= 0 && z < nz && in0 ? pl[0] : 0.0, et);
-        q1[j] = ix_digits(z >= 0 && z < nz && in1 ? pl[1] : 0.0, et);
+        const bool okz = z >= 0 && z < nz;
+        q[j] = top_split(make_double2(okz && in0 ? pl[0] : 0.0, okz && in1 ? pl[1] : 0.0), lo, qt[j]);
     }
-    asm volatile("cp.async.wait_group 2;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
     for (int k = 0; k < kHalf; ++k) split(k, k);
     __syncthreads();
     const double cf = s_cf;
-#pragma unroll
-    for (int k = 0; k < kHalf; ++k) {
-        const int4 hv = *reinterpret_cast<const int4*>(ring + k * kIxPts + ctr);
-        q0[kHalf + k] = make_int2(hv.x, hv.y);
-        q1[kHalf + k] = make_int2(hv.z, hv.w);
-    }
     int slot = 0;   // of plane z0 + k
-    for (int k0 = 0; k0 < nzt; k0 += kZU) {
+    for (int k0 = 0; k0 < nzt; k0 += kHZU) {
 #pragma unroll
-        for (int u = 0; u < kZU; ++u) {
+        for (int u = 0; u < kHZU; ++u) {
             const int k = k0 + u;
             if (k >= nzt) break;
-            // the slot of plane k + 8 held plane k - 2, which every thread has finished
-            if (k + 2 < nzt) copy(k + kHalf + 2, ix_slot(slot, kHalf + 2));
+            // the slot of plane k + 7 held plane k - 2, which every thread has finished
+            if (k + 1 < nzt) copy(k + kHalf + 1, ix_slot<kHRing>(slot, kHalf + 1));
             cp_async_commit();
-            asm volatile("cp.async.wait_group 2;" ::: "memory");
-            const int hslot = ix_slot(slot, kHalf);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            const int hslot = ix_slot<kHRing>(slot, kHalf);
             split(k + kHalf, hslot);
             // psi and the potential at the plane this step computes
             double uc[2] = {0.0, 0.0}, va[2] = {0.0, 0.0}, vb[2] = {0.0, 0.0};
@@ -237,35 +263,52 @@ __global__ void __launch_bounds__(256, 2) k_hamiltonian_ix(const BlkDesc* __rest
                     }
             }
             __syncthreads();   // plane k + 6 is split, every thread has finished plane k - 1
-            {
-                const int4 hv = *reinterpret_cast<const int4*>(ring + hslot * kIxPts + ctr);
-                q0[u + 2 * kHalf] = make_int2(hv.x, hv.y);
-                q1[u + 2 * kHalf] = make_int2(hv.z, hv.w);
-            }
-            const int2* const pc = ring + slot * kIxPts + ctr;
-            slot = ix_slot(slot, 1);
-            int2 xw[2 * kHalf + 2];   // columns -6 .. 7 of the row
+            const HPair* const pc = ring + slot * kIxPairs + ctr;
+            const unsigned* const tc = tops + slot * kIxPairs + ctr;
+            HPair xw[kHalf + 1];   // columns -6 .. 7 of the row
+            unsigned xt[kHalf + 1];
 #pragma unroll
             for (int k2 = 0; k2 < kHalf + 1; ++k2) {
-                const int4 v = *reinterpret_cast<const int4*>(pc - kHalf + 2 * k2);
-                xw[2 * k2] = make_int2(v.x, v.y);
-                xw[2 * k2 + 1] = make_int2(v.z, v.w);
+                xw[k2] = pc[k2 - kHalf / 2];
+                xt[k2] = tc[k2 - kHalf / 2];
             }
-            const int2 c0 = q0[u + kHalf], c1 = q1[u + kHalf];
-            long long H0 = (long long)kWc * c0.x, L0 = (long long)kWc * c0.y;
-            long long H1 = (long long)kWc * c1.x, L1 = (long long)kWc * c1.y;
+            auto xh = [&](int c) { return (c & 1) ? xw[c >> 1].h.y : xw[c >> 1].h.x; };
+            auto xl = [&](int c) { return (c & 1) ? xw[c >> 1].l.y : xw[c >> 1].l.x; };
+            auto xtop = [&](int c) { return (c & 1) ? __byte_perm(xt[c >> 1], xt[(c >> 1) + 1], 0x5432) : xt[c >> 1]; };
+            // centre, then the distances: sums and products exact in (Sh, errors), the rest in Sl
+            const HPair c0 = xw[kHalf / 2];
+            q[u + kHalf] = c0;
+            qt[u + kHalf] = xt[kHalf / 2];
+            long long I0 = (long long)kWc * (int)(xt[kHalf / 2] & 0xffffu), I1 = (long long)kWc * (int)(xt[kHalf / 2] >> 16);
+            const float2 wc = make_float2((float)kWc, (float)kWc);
+            float2 Sh = __fmul2_rn(wc, c0.h);
+            float2 Sl = __ffma2_rn(wc, c0.l, __ffma2_rn(wc, c0.h, make_float2(-Sh.x, -Sh.y)));
 #pragma unroll
             for (int m = 1; m <= kHalf; ++m) {
-                const int4 uu = *reinterpret_cast<const int4*>(pc - m * kPX);
-                const int4 ww = *reinterpret_cast<const int4*>(pc + m * kPX);
-                const int2 a0 = q0[u + kHalf - m], b0 = q0[u + kHalf + m];
-                const int2 a1 = q1[u + kHalf - m], b1 = q1[u + kHalf + m];
-                H0 += (long long)kW[m] * (xw[kHalf - m].x + xw[kHalf + m].x + uu.x + ww.x + a0.x + b0.x);
-                L0 += (long long)kW[m] * (xw[kHalf - m].y + xw[kHalf + m].y + uu.y + ww.y + a0.y + b0.y);
-                H1 += (long long)kW[m] * (xw[kHalf + 1 - m].x + xw[kHalf + 1 + m].x + uu.z + ww.z + a1.x + b1.x);
-                L1 += (long long)kW[m] * (xw[kHalf + 1 - m].y + xw[kHalf + 1 + m].y + uu.w + ww.w + a1.y + b1.y);
+                // x: one lane at a time (at odd distances the neighbours are no pairs)
+                float2 e0, e1, e2, e3, e4, e5, sx;
+                sx.x = two_sum(xh(kHalf - m), xh(kHalf + m), e0.x);
+                sx.y = two_sum(xh(kHalf + 1 - m), xh(kHalf + 1 + m), e0.y);
+                const float2 lx = make_float2(xl(kHalf - m) + xl(kHalf + m), xl(kHalf + 1 - m) + xl(kHalf + 1 + m));
+                const unsigned tx2 = xtop(kHalf - m) + xtop(kHalf + m);
+                const HPair ya = pc[-m * (kPX / 2)], yb = pc[m * (kPX / 2)];
+                const int zs = ix_slot<kHRing>(slot, m) * kIxPairs + ctr;
+                const HPair za = q[u + kHalf - m], zb = ring[zs];
+                const unsigned t = tx2 + (tc[-m * (kPX / 2)] + tc[m * (kPX / 2)]) + (qt[u + kHalf - m] + tops[zs]);
+                I0 += (long long)kW[m] * (int)(t & 0xffffu);
+                I1 += (long long)kW[m] * (int)(t >> 16);
+                const float2 sy2 = two_sum2(ya.h, yb.h, e1), sz2 = two_sum2(za.h, zb.h, e2);
+                const float2 s = two_sum2(two_sum2(sx, sy2, e3), sz2, e4);
+                float2 l = __fadd2_rn(__fadd2_rn(lx, __fadd2_rn(ya.l, yb.l)), __fadd2_rn(za.l, zb.l));
+                l = __fadd2_rn(l, __fadd2_rn(__fadd2_rn(e0, e1), __fadd2_rn(e2, __fadd2_rn(e3, e4))));
+                const float2 w = make_float2((float)kW[m], (float)kW[m]);
+                const float2 p = __fmul2_rn(w, s);
+                const float2 ep = __ffma2_rn(w, s, make_float2(-p.x, -p.y));
+                Sh = two_sum2(Sh, p, e5);
+                Sl = __fadd2_rn(__ffma2_rn(w, l, Sl), __fadd2_rn(ep, e5));
             }
-            double r[2] = {ix_to_double(H0, L0) * cf, ix_to_double(H1, L1) * cf};
+            slot = ix_slot<kHRing>(slot, 1);
+            double r[2] = {top_join(I0, Sh.x, Sl.x, cf), top_join(I1, Sh.y, Sl.y, cf)};
             if (pot) {
 #pragma unroll
                 for (int a = 0; a < 2; ++a) r[a] = fma(vloc && vavg ? va[a] + vb[a] : (vloc ? va[a] : vb[a]), uc[a], r[a]);
@@ -278,8 +321,11 @@ __global__ void __launch_bounds__(256, 2) k_hamiltonian_ix(const BlkDesc* __rest
                 if (in1) o[1] = r[1];
             }
         }
-        ix_shift(q0);
-        ix_shift(q1);
+#pragma unroll
+        for (int j = 0; j < kHalf; ++j) {
+            q[j] = q[j + kHZU];
+            qt[j] = qt[j + kHZU];
+        }
     }
     if (s_bad) {   // NaN wherever a tap reads a value out of range (the float-float sweep did so too)
         for (int z = P.z0; z < P.z1; ++z)
@@ -349,7 +395,7 @@ void launch_hamiltonian(const flosic_ctx* c, const double* psi, const double* vl
         k_tile_exp<<<(unsigned)M.ntiles[0], tb, 0, s>>>(c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, psi,
                                                                  c->ws.texp);
         note_launch((flosic_ctx*)c);
-        k_hamiltonian_ix<<<(unsigned)M.ntiles[0], dim3(kTileX / 2, kTileY), kHSmem, s>>>(
+        k_hamiltonian_mixed<<<(unsigned)M.ntiles[0], dim3(kTileX / 2, kTileY), kHSmem, s>>>(
             c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, psi, vloc, vavg, c->ws.texp, hpsi);
     } else
         k_hamiltonian64<<<(unsigned)M.ntiles[0], tb, 0, s>>>(c->d_blk, M.d_lvl[0], M.d_tiles[0], c->d_orb_blk, psi,
@@ -362,7 +408,7 @@ cudaError_t upload_hamiltonian_constants() {
     stencil_weights(w);
     const cudaError_t e = cudaMemcpyToSymbol(c_w64, w, sizeof(w));
     if (e != cudaSuccess) return e;
-    return ensure_dyn_smem((const void*)k_hamiltonian_ix, kHSmem);
+    return ensure_dyn_smem((const void*)k_hamiltonian_mixed, kHSmem);
 }
 
 }  // namespace flosic

@@ -1,6 +1,6 @@
-// Exact integer sums of the 12th-order stencil (Sec. II.A: high-order centred
-// finite differences), shared by the refinement update and the
-// mixed-precision Hamiltonian apply.
+// The 12th-order stencil (Sec. II.A: high-order centred finite differences) in
+// integer weights, and the staging of its planes, shared by the refinement update
+// and the mixed-precision Hamiltonian apply.
 #pragma once
 #include <cmath>
 
@@ -13,9 +13,8 @@ namespace flosic {
 // 2 (-1)^(m+1) (6!)^2 / (m^2 (6-m)! (6+m)!), w_0 = -2 sum w_m) are rationals
 // whose common denominator is 831600, so W_m = 831600 w_m are integers and
 // h^2 Delta_h u = (1 / 831600) sum_m W_m (sum of the six neighbours at
-// distance m).  A field in fixed point (an integer per point, or two digits)
-// is summed and weighted without rounding: six values of at most 2^28 stay
-// below 2^31, the weighted sum below 2^53.
+// distance m).  An integer field is summed and weighted without rounding: six
+// values of at most 2^28 stay below 2^31, the weighted sum below 2^53.
 // ---------------------------------------------------------------------------
 constexpr long long kW12Den = 831600;
 
@@ -82,7 +81,8 @@ constexpr int kIxPts = kPX * kPY;                    // points of a staged plane
 constexpr int kIxPairs = kIxPts / 2;
 constexpr int kIxU = (kIxPairs + 255) / 256;         // pairs per thread
 constexpr int kIxRing = 10;
-__device__ __forceinline__ int ix_slot(int s, int d) { return s + d >= kIxRing ? s + d - kIxRing : s + d; }   // d planes on
+template <int kRing = kIxRing>
+__device__ __forceinline__ int ix_slot(int s, int d) { return s + d >= kRing ? s + d - kRing : s + d; }   // d planes on
 
 template <int kBytes>
 __device__ __forceinline__ void cp_async(void* dst, const void* src, int bytes) {   // the rest of kBytes is zeroed
