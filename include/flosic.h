@@ -29,6 +29,9 @@
  *    system.  flosic_layout() returns every packed size.
  *  - Device arrays need the alignment of their elements only; the wide accesses
  *    of arrays on 16-byte boundaries give way to single ones otherwise.
+ *  - The order of partial sums follows the whole batch and the GPU's size (tile
+ *    depths, splits of the contractions), so a system's last bits may differ
+ *    between batches; for one context they are the same on every call.
  *  - Every call is asynchronous on `stream` (a cudaStream_t, passed as
  *    void*), except that calls whose result can fail on the device
  *    (flosic_build_flos: ILLCOND/NONFINITE, flosic_orbital_poisson: NOCONV)
