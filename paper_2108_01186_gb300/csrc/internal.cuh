@@ -587,11 +587,6 @@ __device__ __forceinline__ ff ff_sum6(ff a, ff b, ff c, ff d, ff e, ff f) {
     err += ((a.l + b.l) + (c.l + d.l)) + (e.l + f.l);
     return ff_quick(s.h, err);
 }
-// a + b with b a plain float (two-sum, then renormalise)
-__device__ __forceinline__ ff ff_addf(ff a, float b) {
-    const ff s = ff_two_sum(a.h, b);
-    return ff_quick(s.h, s.l + a.l);
-}
 // Running sum of pairs (th, tl) with |tl| small against |th|: exact
 // two-sum of the high parts, the low parts and its rounding error gathered in
 // a.l without renormalising; after n terms the error is ~n 2^-48 sum |terms|
@@ -620,12 +615,6 @@ __device__ __forceinline__ ff warp_sum(ff v) {
 // index of point (x, y, z) of orbital i of block B in the Kronecker solver's padded arrays
 __device__ __forceinline__ long long pad_index(const BlkDesc& B, int i, int x, int y, int z) {
     return B.poff + (long long)i * B.Gp + ((long long)z * B.p[1] + y) * B.p[0] + x;
-}
-
-__device__ __forceinline__ int find_block(const BlkDesc* blk, int nblk, int orb) {
-    int b = 0;
-    while (b + 1 < nblk && blk[b + 1].orb0 <= orb) ++b;
-    return b;
 }
 
 // ---- 3-D tiles of one orbital (x0, y0, z0; kTileX x kTileY x kTileZ) ----

@@ -17,21 +17,23 @@
 // p (kron_pad: a multiple of 4, p = n when n is a multiple of 8), in every
 // layout, so that each row starts on a 16-byte boundary and any side will
 // do: the even modes of a line sit at [0, ns), the odd ones at [ns4, ns4 +
-// na) with ns4 = ns rounded up to 4.  Padding rows carry finite garbage into
-// padding rows only, and padding elements of a line are masked when the line
-// is read.  Every input row is a contiguous run that one tiled bulk copy
+// na) with ns4 = ns rounded up to 4.  The padding is never
+// initialised and may hold anything, NaN too: a row only ever reaches its own
+// results (padding rows end in padding rows), and the padding elements of a line
+// are dropped by selection, not by a product, when the line is read and when
+// results are stored.  Every input row is a contiguous run that one tiled bulk copy
 // (TMA, 128-byte swizzle) brings to shared memory; every output store is
 // coalesced (the 32 lanes of a warp own 32 consecutive rows).
 //
-// One CTA per SM (13 warps) streams tiles of 128 rows.  The copy engine
+// One CTA per SM (14 warps) streams tiles of 128 rows.  The copy engine
 // delivers a tile's rows (float32) into a ring of 32-point boxes, up to two
 // tiles ahead.  Eight converter warps fold each row into its even and odd
 // halves (s_k = v_k + v_{n-1-k}, a_k = v_k - v_{n-1-k}: T_d commutes with the
 // reflection, so the transform splits into two half-size products) and write
 // each half as three bf16 terms (v = v1 + v2 + v3, ~24 significant bits)
 // straight into tensor memory, the MMAs' A operand (row i in lane i); the
-// split matrices stay in shared memory (B operand, K-major).  A control warp
-// issues the copies and the MMAs: per unit of 32 modes of one half, the six
+// split matrices stay in shared memory (B operand, K-major).  One warp issues
+// the copies, another the MMAs: per unit of 32 modes of one half, the six
 // split products v_i w_j with i + j <= 2, the v1 w1 product into its own
 // accumulator and the five smaller ones into a second.  Units rotate through
 // a ring of accumulators, so the MMAs run ahead while the four epilogue

@@ -19,30 +19,18 @@
 // loses most of its strength on grids such as 128^3.  Restriction is full
 // weighting (1/4, 1/2, 1/4 per direction) = (1/8) P^T with P trilinear
 // interpolation.  Smoother: one damped-Jacobi sweep before and after
-// (omega = 0.8); coarsest level: 40 damped-Jacobi sweeps from zero.  Every piece is symmetric and the smoother converges in the A2
-// norm, so the V-cycle is a symmetric positive definite operator.
+// (omega = 0.8); coarsest level: 40 damped-Jacobi sweeps from zero.  Every
+// piece is symmetric and the smoother converges in the A2 norm, so the V-cycle
+// is a symmetric positive definite operator.
 //
-// Kernels work on per-level tables of 3-D tiles (one CTA per 32 x 16 x 32
-// tile of one orbital) so that all orbitals of all systems run in one launch
+// Kernels work on per-level tables of 3-D tiles (one CTA of 32 x 8 threads per
+// 32 x 16 column of one orbital, as many planes deep as tile_depth and
+// tile_split say; neighbours come through L1) so that all orbitals of all systems run in one launch
 // per level; the levels small enough for shared memory run in one launch
 // together (k_mg_coarse).
 #include "internal.cuh"
 
 namespace flosic {
-
-// Each CTA (32 x 8 threads) owns a 32 x 16 x 32 tile of one orbital on one
-// level: thread (tx, ty) handles the points (x0+tx, y0+ty+8k, z), k = 0, 1,
-// for every plane z of the tile.  Neighbours come through L1.
-template <class Body>
-__device__ __forceinline__ void for_tile_points(const LvlDesc& D, const TilePos& P, Body body) {
-    const int x = P.x0 + threadIdx.x;
-    if (x >= D.nx) return;
-    for (int k = 0; k < 2; ++k) {
-        const int y = P.y0 + threadIdx.y + k * (kTileY / 2);
-        if (y >= D.ny) continue;
-        for (int z = P.z0; z < P.z1; ++z) body(x, y, z, ((long long)z * D.ny + y) * D.nx + x);
-    }
-}
 
 // sum of the six neighbours (zero outside)
 template <class T>

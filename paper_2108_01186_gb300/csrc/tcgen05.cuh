@@ -158,21 +158,6 @@ __device__ __forceinline__ void tmem_st4(uint32_t taddr, uint32_t v0, uint32_t v
 // this thread's tensor-memory stores have completed
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// 2-D tiled bulk copy shared -> global (completion tracked by bulk groups)
-__device__ __forceinline__ void tc_tma_store_2d(const CUtensorMap* map, int c0, int c1, const void* src) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
-                     (unsigned long long)map),
-                 "r"(c0), "r"(c1), "r"(tc_smem_addr(src))
-                 : "memory");
-}
-__device__ __forceinline__ void tc_bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// at most one committed bulk group still reads shared memory
-__device__ __forceinline__ void tc_bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-// no committed bulk group still reads shared memory
-__device__ __forceinline__ void tc_bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// every committed bulk group has completed
-__device__ __forceinline__ void tc_bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 // 32 consecutive columns of this warp's 32 tensor-memory lanes (one column per register)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* out) {
     uint32_t v[32];
@@ -211,25 +196,10 @@ __device__ __forceinline__ void tc_mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc_smem_addr(bar)) : "memory");
 }
 
-// bounded wait that also gives up as soon as *abort (shared) becomes nonzero
-__device__ __forceinline__ bool tc_mbar_wait_or_abort(uint64_t* bar, uint32_t parity, const volatile int* abort) {
-    for (long long i = 0; i < kTcWaitLimit; ++i) {
-        uint32_t ok;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(ok)
-            : "r"(tc_smem_addr(bar)), "r"(parity)
-            : "memory");
-        if (ok) return true;
-        if (*abort) return false;
-    }
-    return false;
-}
-
-// As tc_mbar_wait_or_abort, but each poll may suspend the thread for up to
-// about a microsecond (it resumes as soon as the phase completes), so a
-// waiting warp takes almost no issue slots; gives up after about two
-// seconds.
+// Bounded wait that also gives up as soon as *abort (shared) becomes nonzero.
+// Each poll may suspend the thread for up to about a microsecond (it resumes as
+// soon as the phase completes), so a waiting warp takes almost no issue slots;
+// gives up after about two seconds.
 __device__ __forceinline__ bool tc_mbar_sleep_or_abort(uint64_t* bar, uint32_t parity, const volatile int* abort) {
     for (int i = 0; i < (1 << 21); ++i) {
         uint32_t ok;
