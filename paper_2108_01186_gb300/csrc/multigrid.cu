@@ -325,16 +325,16 @@ __global__ void __launch_bounds__(256) k_mg_prolong(const BlkDesc* __restrict__ 
     }
     const long long sy = F.nx, sz = (long long)F.nx * F.ny;
     const T d = oh2 * T(1.0 / 6.0);
-    const int nzp = (P.z1 - P.z0 + 1) >> 1;                 // z pairs in the tile
+    const int ze = P.z0 & ~1, nzp = (P.z1 - ze + 1) >> 1;   // z pairs that meet the tile (it may start on an odd plane)
     for (int w = linear_tid(); w < 8 * (kTileY / 2) * nzp; w += 256) {
         const int xg = w & 7, rest = w >> 3;
         const int yp = rest % (kTileY / 2), zp = rest / (kTileY / 2);
-        const int x = P.x0 + 4 * xg, y = P.y0 + 2 * yp, z = P.z0 + 2 * zp;
+        const int x = P.x0 + 4 * xg, y = P.y0 + 2 * yp, z = ze + 2 * zp;
         if (x >= F.nx || y >= F.ny) continue;
-        if (y + 1 >= F.ny || z + 1 >= P.z1) {               // ragged edge: row by row
+        if (y + 1 >= F.ny || z < P.z0 || z + 1 >= P.z1) {   // ragged edge: row by row
             for (int c = 0; c < 2; ++c)
                 for (int b = 0; b < 2; ++b)
-                    if (y + b < F.ny && z + c < P.z1)
+                    if (y + b < F.ny && z + c >= P.z0 && z + c < P.z1)
                         prolong_row<T>(F, C, eb, r, t, oh2, x, y + b, z + c,
                                        P.base + (z + c) * sz + (y + b) * sy + x, 4);
             continue;
