@@ -29,8 +29,9 @@ static inline cudaError_t upload_ffsweep_weights() {
 }
 
 // load(g) -> float2 pair of the operand at flat index g (only called for
-// points inside the grid); epi(g, centre, lap) with lap = h^2 Delta_h u at g
-// as a pair, called for every point of the tile inside the grid.
+// points inside the grid); epi(g, k, z, centre, lap) with lap = h^2 Delta_h u
+// at g as a pair, called for every point of the tile inside the grid: plane z of
+// the thread's column k (x0 + tx, y0 + ty + 8 k).
 // The seven weighted terms are accumulated with the two-sum of the high parts
 // and a plain sum of the low parts (error ~ eps^2 times the sum of the terms'
 // magnitudes, ~1e-12 of the result for the smooth potentials of the residual).
@@ -110,7 +111,7 @@ __device__ __forceinline__ void ff_sweep12(const LvlDesc& D, const TilePos& P, L
                 const ff s2 = ff_two_sum(acc.h, tm.h);
                 acc = ff_quick(s2.h, s2.l + (acc.l + tm.l));
             }
-            if (in[k]) epi(P.base + z * sz + cc[k], qk[kHalf], acc);
+            if (in[k]) epi(P.base + z * sz + cc[k], k, z, qk[kHalf], acc);
         }
         __syncthreads();
 #pragma unroll
