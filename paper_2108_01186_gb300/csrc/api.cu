@@ -573,7 +573,7 @@ int flosic_create(flosic_ctx** out, const flosic_system* sys, int nsys, const fl
     const long long nparts = chunk > M.ntiles[0] ? chunk : M.ntiles[0];
     if (o.solver == FLOSIC_SOLVER_AAR) A(&w.aar_part, aar_part_elems(M.ntiles[0]));
     A(&w.mom_part, 10 * nparts);
-    if (o.precision == FLOSIC_MIXED) A(&w.texp, M.ntiles[0]);
+    if (o.precision == FLOSIC_MIXED) { A(&w.texp, M.ntiles[0]); A(&w.vsum, c->vavg_elems); }
     A(&g.part, nparts); A(&g.part2, nparts); A(&g.count, orb); A(&g.active, orb); A(&g.oactive, orb);
     A(&g.iters, orb); A(&g.n_active, 1); A(&g.n_oactive, 1); A(&g.conv, orb); A(&g.prof_bytes, 1);
     A(&g.dmax, orb); A(&g.xz, orb);

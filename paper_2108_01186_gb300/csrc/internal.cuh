@@ -202,6 +202,7 @@ struct Workspace {
     float *z32, *p32b;               // multigrid PCG (FP32)
     CgState cg;
     int* texp;             // [level-0 tiles] largest exponent of the operand per tile (mixed Hamiltonian apply)
+    double* vsum;          // [sum G over blocks] both its potentials added up
 };
 
 struct Multigrid {

@@ -115,12 +115,17 @@ struct IxStage {
             if (iny && px >= 0 && px < D.nx) f |= 4;
             if (iny && p1 >= 0 && p1 < D.nx) f |= 8;
             if (p1 != px + 1) f |= 16;
-            off[j] = py * pitch + px;
+            off[j] = (f & 12) ? py * pitch + px : 0;
             fl |= f << (8 * j);
         }
     }
     // is pair j read by a tap (full: the plane is one of the tile's)?
     __device__ __forceinline__ bool wants(int j, bool full) const { return (fl >> (8 * j)) & (full ? 1u : 2u); }
+    // the same where both points are inside or neither is, and always aligned to their pair
+    template <class T>
+    __device__ __forceinline__ void copy_pair(int j, void* to, const T* plane, bool okz) const {
+        cp_async<2 * sizeof(T)>(to, plane + off[j], okz && (fl & (4u << (8 * j))) ? 2 * (int)sizeof(T) : 0);
+    }
     // pair j of the plane to `to`; vec: the points are always neighbours and both aligned to their pair
     template <class T>
     __device__ __forceinline__ void copy(int j, void* to, const T* plane, bool okz, bool vec, int nx) const {
