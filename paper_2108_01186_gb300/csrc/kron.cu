@@ -131,11 +131,11 @@ struct KronArgs {
 //   x: lines are grid rows (y, z), tile q = rows q*C .. q*C+C-1 (a contiguous run of C*nx values)
 //   y: lines are (x, z) columns at fixed z, tile q = (z, x-group)
 //   z: lines are xy points, tile q = xy points q*C .. q*C+C-1
-// (only blocks on the tensor cores have padded sides)
+// (rows and xy points run over the padded sides of the arrays)
 __device__ __forceinline__ int pass_groups(const BlkDesc& B, int axis) {
-    if (axis == 0) return (B.ny * B.nz + kKronCols - 1) / kKronCols;
+    if (axis == 0) return (B.p[1] * B.nz + kKronCols - 1) / kKronCols;
     if (axis == 1) return B.nz * ((B.nx + kKronCols - 1) / kKronCols);
-    return (B.nx * B.ny + kKronCols - 1) / kKronCols;
+    return (B.p[0] * B.ny + kKronCols - 1) / kKronCols;
 }
 
 // Addressing of one tile: element (j, c) = position j along line c lies at
@@ -147,26 +147,26 @@ struct Tile {
 
 __device__ __forceinline__ Tile tile_of(const BlkDesc& B, int axis, int i_orb, int q) {
     Tile t;
-    const long long base = B.poff + (long long)i_orb * B.G;
-    const long long sxy = (long long)B.nx * B.ny;
+    const long long base = B.poff + (long long)i_orb * B.Gp;
+    const long long px = B.p[0], sxy = px * B.p[1];
     t.q = q;
     if (axis == 0) {
-        t.cbase = base + (long long)q * kKronCols * B.nx;
-        t.cstride = B.nx;
+        t.cbase = base + (long long)q * kKronCols * px;
+        t.cstride = px;
         t.jstride = 1;
-        t.ncol = min(kKronCols, B.ny * B.nz - q * kKronCols);
+        t.ncol = min(kKronCols, B.p[1] * B.nz - q * kKronCols);
     } else if (axis == 1) {
         const int gx = (B.nx + kKronCols - 1) / kKronCols;
         const int zi = q / gx, xg = q - zi * gx;
         t.cbase = base + (long long)zi * sxy + (long long)xg * kKronCols;
         t.cstride = 1;
-        t.jstride = B.nx;
+        t.jstride = px;
         t.ncol = min(kKronCols, B.nx - xg * kKronCols);
     } else {
         t.cbase = base + (long long)q * kKronCols;
         t.cstride = 1;
         t.jstride = sxy;
-        t.ncol = (int)min((long long)kKronCols, sxy - (long long)q * kKronCols);
+        t.ncol = (int)min((long long)kKronCols, px * B.ny - (long long)q * kKronCols);
     }
     return t;
 }
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(2 * kKronMaxN) k_kron_pass(KronArgs a, long lo
         if (!a.inverse) {
             if (comp) {
                 if (a.scale) {   // forward z pass: column c is the xy mode (t % nx, t / nx)
-                    const long long sxy = (long long)B.nx * B.ny;
+                    const long long sxy = (long long)B.p[0] * B.ny;
                     const float* lx = a.lam + B.kl[0];
                     const float* ly = a.lam + B.kl[1];
                     const float* lz = a.lam + B.kl[2];
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(2 * kKronMaxN) k_kron_pass(KronArgs a, long lo
                     for (int v = 0; v < 4; ++v) {
                         const long long tt = (long long)t.q * kKronCols + c0 + v;
                         const int ti = (int)(tt < sxy ? tt : 0);
-                        const int yi = ti / B.nx, xi = ti - yi * B.nx;
+                        const int yi = ti / B.p[0], xi = ti - yi * B.p[0];
                         lxy[v] = lx[xi] + ly[yi];
                     }
 #pragma unroll
@@ -642,9 +642,9 @@ cudaError_t setup_kron(flosic_ctx* c) {
             const BlkDesc& B = c->blk[b];
             items[(size_t)d * (c->nblk + 1) + b] = acc;
             long long g;
-            if (d == 0) g = (B.ny * (long long)B.nz + kKronCols - 1) / kKronCols;
+            if (d == 0) g = (B.p[1] * (long long)B.nz + kKronCols - 1) / kKronCols;
             else if (d == 1) g = (long long)B.nz * ((B.nx + kKronCols - 1) / kKronCols);
-            else g = ((long long)B.nx * B.ny + kKronCols - 1) / kKronCols;
+            else g = ((long long)B.p[0] * B.ny + kKronCols - 1) / kKronCols;
             if (!B.tc) acc += g * B.N;   // tensor-core blocks take no tiles of this kernel
             const int n = d == 0 ? B.nx : (d == 1 ? B.ny : B.nz);
             nmax = n > nmax ? n : nmax;
@@ -678,13 +678,13 @@ cudaError_t setup_kron(flosic_ctx* c) {
 }
 
 // Autotuner of the transforms: per distinct shape (nx, ny, nz, N, periodic
-// sides) of the blocks whose sides are multiples of 8 up to 128 (the others
-// that may take the tensor cores always do, see kron_tc_eligible), one inner
-// solve of one block of that shape is timed (CUDA events, after a warm-up
-// solve, three solves averaged, zero input: the transforms' cost does not
-// depend on the values) with every qualifying block on the tensor cores and
-// again with every one on the CUDA cores; each shape keeps the faster, and the
-// solver is planned once more with those choices.  Runs once, at context creation.
+// sides) of the blocks whose sides are multiples of 8 up to 128 (the padded
+// shapes always take the tensor cores), one inner solve of
+// one block of that shape is timed (CUDA events, after a warm-up solve, three
+// solves averaged, zero input: the transforms' cost does not depend on the
+// values) with every qualifying block on the tensor cores and again with
+// every block on the CUDA cores; each shape keeps the faster, and the solver
+// is planned once more with those choices.  Runs once, at context creation.
 cudaError_t kron_autotune(flosic_ctx* c) {
     KronPlan& K = c->kron;
     std::map<std::array<long long, 5>, std::vector<int>> groups;
@@ -714,9 +714,7 @@ cudaError_t kron_autotune(flosic_ctx* c) {
     if (e == cudaSuccess) e = cudaMemcpy(dflags, hflags.data(), sizeof(int) * hflags.size(), cudaMemcpyHostToDevice);
     std::vector<float> t_tc(groups.size(), 0.f), t_cc(groups.size(), 0.f);
     auto plan = [&](int force) {   // force 1: every qualifying block on the tensor cores; 0: none
-        K.tc_force.assign((size_t)c->nblk, 1);
-        for (const auto& g : groups)
-            for (int b : g.second) K.tc_force[(size_t)b] = force;
+        K.tc_force.assign((size_t)c->nblk, force);
         cudaError_t r = setup_kron(c);
         if (r == cudaSuccess)
             r = cudaMemcpy(c->d_blk, c->blk.data(), sizeof(BlkDesc) * c->nblk, cudaMemcpyHostToDevice);
