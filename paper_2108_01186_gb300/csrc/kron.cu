@@ -679,12 +679,16 @@ cudaError_t setup_kron(flosic_ctx* c) {
 
 // Autotuner of the transforms: per distinct shape (nx, ny, nz, N, periodic
 // sides) of the blocks whose sides are multiples of 8 up to 128 (the padded
-// shapes always take the tensor cores), one inner solve of
+// shapes always take the tensor cores, see kron_tc_eligible), one inner solve of
 // one block of that shape is timed (CUDA events, after a warm-up solve, three
 // solves averaged, zero input: the transforms' cost does not depend on the
 // values) with every qualifying block on the tensor cores and again with
 // every block on the CUDA cores; each shape keeps the faster, and the solver
-// is planned once more with those choices.  Runs once, at context creation.
+// is planned once more with those choices.  Both plans list every qualifying
+// block, the padded ones too: the block timed lies among the others' idle tiles
+// either way.  (With the padded blocks on the tensor cores in both, a batch of seven
+// molecules had a wrong choice, its solves 3.83 -> 4.25 ms.)  Runs once, at context
+// creation.
 cudaError_t kron_autotune(flosic_ctx* c) {
     KronPlan& K = c->kron;
     std::map<std::array<long long, 5>, std::vector<int>> groups;

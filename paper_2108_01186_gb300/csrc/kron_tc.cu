@@ -779,11 +779,16 @@ int kron_pad(int n) {
     return (ns4 + n / 2 + 3) & ~3;
 }
 
-// Sides that are multiples of 8 up to 128 need no padding and take the
-// tensor cores at any size; other sides do from 32 points up to the 192 whose
-// matrices fit in shared memory (below 32 the CUDA-core tiles are as fast and
-// need no padding).  Measured per solve: 117^3 x 20 0.44 ms here, 1.35 ms on the
-// CUDA cores; 192^3 x 24 1.82 and 7.35 ms.
+// Sides that are multiples of 8 up to 128 need no padding and may take the
+// tensor cores at any size (the autotuner decides, kron.cu); other sides do from
+// 32 points up to the 192 whose matrices fit in shared memory (below 32 the
+// CUDA-core tiles are as fast and need no padding).  Measured per inner solve:
+// 117^3 x 20 0.44 ms here, 1.35 ms on the CUDA cores; 192^3 x 24 1.82 and 7.35 ms.
+// Whole Poisson solves, here and there: 33^3 x 1 293 and 325 us, x 50 563 and 693;
+// 44^3 x 5 316 and 372; 61^3 x 2 309 and 365; 90 x 36 x 33 x 1 308 and 352;
+// 75^3 x 10 699 and 960; 140^3 x 1 637 and 893 (78 shapes with sides of 33 to 192
+// points and 1 to 50 orbitals: always the faster, so these are not timed at
+// creation).
 bool kron_tc_eligible(const BlkDesc& B) {
     const int nd[3] = {B.nx, B.ny, B.nz};
     bool general = true;
