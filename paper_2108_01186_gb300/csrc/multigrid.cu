@@ -164,21 +164,26 @@ __global__ void __launch_bounds__(256) k_mg_restrict(const BlkDesc* __restrict__
     const T* fb = sf + fbase;
     const long long fy = F.nx, fz = (long long)F.nx * F.ny;
     const bool fvec = (F.nx % (2 * V) == 0) && (fbase % (2 * V) == 0);
+    // float64: the nine fine rows' loads in flight together (48^3 x 40 89 against 97 us,
+    // 64^3 x 6 19.6 and 21.0).  float32 takes the rows one after the other: nine at once
+    // cost registers (128^3 x 24 68 against 56 us, 117^3 x 16 124 and 72, 64^3 x 10 8.2
+    // and 6.1, 33^3 x 5 7.7 and 5.9)
+    constexpr bool kAhead = sizeof(T) == sizeof(double);
+    constexpr int kU = kAhead ? 3 : 1;
     tile_rows<T>(C, P, [&](int X, int Y, int Z, long long g, int n) {
         T acc[V];
 #pragma unroll
         for (int k = 0; k < V; ++k) acc[k] = T(0);
         const int xf0 = 2 * X;
-        // the nine fine rows unrolled: their loads are independent and in flight
-        // together (rows past the grid count as zero)
-#pragma unroll
+#pragma unroll kU
         for (int c = 0; c < 3; ++c) {
             const int zf = 2 * Z + c;
             const T wc = (c == 1) ? T(0.5) : T(0.25);
-#pragma unroll
+#pragma unroll kU
             for (int b = 0; b < 3; ++b) {
                 const int yf = 2 * Y + b;
-                const bool ok = zf < F.nz && yf < F.ny;
+                const bool ok = zf < F.nz && yf < F.ny;   // rows past the grid count as zero
+                if (!kAhead && !ok) continue;
                 const T w = wc * ((b == 1) ? T(0.5) : T(0.25));
                 const T* row = fb + (ok ? zf * fz + yf * fy : 0);
                 T f[2 * V + 1];
