@@ -673,6 +673,8 @@ int flosic_build_flos(flosic_ctx* c, const double* psi, const double* fods, doub
     int st[4];
     rc = read_status(c, s, st);
     if (rc) return rc;
+    if (st[3])
+        return fail(c, FLOSIC_ERR_CUDA, "a tensor-core completion of the overlap kernel did not arrive (bounded wait expired)");
     if (st[0]) return fail(c, FLOSIC_ERR_NONFINITE, "non-finite value in psi or at a FOD");
     if (st[2]) return fail(c, FLOSIC_ERR_ILLCOND, "Fermi-orbital overlap is near singular (FODs too close?)");
     c->have_forward = true;
@@ -775,6 +777,9 @@ int flosic_sic_backward(flosic_ctx* c, const double* psi, const double* fods, co
         int st[4];
         int rc = read_status(c, s, st);
         if (rc) return rc;
+        if (st[3])
+            return fail(c, FLOSIC_ERR_CUDA,
+                        "a bulk copy or a tensor-core completion of the adjoint Poisson solve did not arrive (bounded wait expired)");
         if (st[1]) return fail(c, FLOSIC_ERR_NOCONV, "adjoint Poisson solve reached max_iter");
         return FLOSIC_OK;
     }

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(256, NB <= 2 ? 2 : 1) k_gram_tc(const BlkDesc*
             for (int j = 0; j < NN; ++j)
                 if (j < N) out[(long long)a * N + j] = acc[j];
         }
-    } else if (!ok && tid == 0) {
+    } else if (!ok && lane == 0) {                   // (any warp: its partial is missing)
         atomicOr(status + 3, 2);                     // an MMA completion did not arrive in time
     }
     tc_fence_before();
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(288, 1) k_gram_async(const BlkDesc* __restrict
                 }
             }
         }
-        if (!ok && tid == 0) atomicOr(status + 3, 2);   // an MMA completion did not arrive in time
+        if (!ok && lane == 0) atomicOr(status + 3, 2);   // an MMA completion did not arrive in time (any warp's)
     }
     tc_fence_before();
     __syncthreads();
